@@ -1907,6 +1907,56 @@ void halo_default(const ConvLayer& L, int& R, int& P, int& ckmax) {
     ckmax = 16;
 }
 
+// Tile of an untuned launch for a layer at (B, W, H): rows R, parity classes P and epilogue
+// warps E.  The chunk width CK and whether the classes run alone (P = 1) or in pairs stay as
+// halo_default chose them: they fix the order in which an accumulator's products are added,
+// so the results do not depend on the choice made here.
+//  - When halo_default's tile gives every SM at most one tile, it stays: smaller tiles would
+//    shorten a frame that has the GPU to itself (256x256: 243 -> 217 us of kernel time), but
+//    take more SM time in all, and frames of several contexts or streams share the SMs
+//    (three contexts: 100.9 -> 103.0 us per frame).
+//  - Else the tile with the least ceil(tiles / SMs) * (accumulators per tile + 1): every tile
+//    costs its accumulators plus about one more for its halo rows and hand-overs, and tiles
+//    are handed out in whole waves.  Ties go to the larger tile.
+//  - TMEM holds two tiles' accumulators (the epilogue overlaps the next tile's MMAs) unless
+//    that leaves fewer than 4 in a concat conv or 2 in another one, i.e. N >= 128 or 256;
+//    then one tile's (each staged weight block feeds twice the pixels: decoder level 2 of a
+//    1080p view, N = 128: 109 us with two buffers, 75 us with one).
+//  - 12 epilogue warps for narrow outputs without pooling (N <= 32: the first conv of 8 1080p
+//    views 328 -> 316 us, the last with its head 328 -> 309 us), else 8.
+//  - Stores go straight to global memory: staging them in shared memory for TMA costs the
+//    pipeline a stage or the epilogue a copy, and lost in every layer but two that it left
+//    unchanged (first conv of a 1080p view: 72 us staged, 54 us direct).
+// False when no tile fits.
+bool halo_pick(const ConvLayer& L, int esize, int ck, int B, int W, int H, int num_sms, int& R, int& P, int& E) {
+    const int N = L.cout, p_default = P;
+    E = !L.cin1 && !L.pool && N <= 32 ? 12 : 8;
+    auto tiles_of = [&](int r, int pp) {
+        const int w = L.cin1 ? W / 2 : W, h = L.cin1 ? H / 2 : H;
+        return (long)B * ((w + 127) / 128) * ((h + r - 1) / r) * (pp ? 4 / pp : 1);
+    };
+    if (tiles_of(R, P) <= num_sms) return 2 * halo_stage_bytes(L, R, P, ck, esize) <= 220u * 1024u;
+    long best = -1;
+    int best_area = 0;
+    const int Ps[3] = {4, 2, 1};
+    for (int pi = 0; pi < (L.cin1 ? 3 : 1); ++pi)
+        for (int r = 8; r >= 1; r /= 2) {
+            const int pp = L.cin1 ? Ps[pi] : 0, area = r * (pp ? pp : 1);
+            if (L.cin1 && ((pp == 1) != (p_default == 1) || !halo_parity_ok(L, pp))) continue;
+            const bool single = N * (L.cin1 ? 4 : 2) > 256;
+            if (area * N > (single ? 512 : 256) || (L.pool && (r & 1))) continue;
+            if (2 * halo_stage_bytes(L, r, pp, ck, esize) > 220u * 1024u) continue;
+            const long cost = (tiles_of(r, pp) + num_sms - 1) / num_sms * (area + 1);
+            if (best < 0 || cost < best || (cost == best && area > best_area)) {
+                best = cost;
+                best_area = area;
+                R = r;
+                P = pp;
+            }
+        }
+    return best >= 0;
+}
+
 // Shared-memory staging of the TMA-store epilogue, bytes per epilogue warp: (pool ? 2 : 1)
 // rows of 32 pixels x N channels of eo bytes, then (pool) 16 pooled pixels of ep bytes, every
 // part 1024-aligned; 0 when the layout has no matching TMA swizzle (row bytes not a power of
@@ -2275,6 +2325,14 @@ bool tc_fused_enc0(const ConvLayer& L0, const ConvLayer& L1, lnr_precision prec,
     return tc_enc0_fused(L0, L1, in, out, pool_out, B, W, H, R, st, ty);
 }
 
+// Whether a test's environment switch asks for one kernel variant everywhere: the untuned
+// choices then step aside.
+bool tc_variant_forced() {
+    static const bool forced = getenv("LNR_CONV_KERNEL") || getenv("LNR_CONV_EPI") || getenv("LNR_CONV_TMA_STORE") ||
+                               getenv("LNR_CONV_TMEM1");
+    return forced;
+}
+
 void tc_conv(const ConvLayer& L, lnr_precision prec, const void* src0, const void* src1, void* out, void* pool_out,
              const float* head_w, const float* head_b, const float* head_wh, const float* head_bh, float* head_out, int B,
              int W, int H, int head_o, cudaStream_t st, const TcConfig* force) {
@@ -2316,7 +2374,12 @@ void tc_conv(const ConvLayer& L, lnr_precision prec, const void* src0, const voi
         if (cfg.mode == 0) {
             halo_default(L, R, P, CK);
             if (ty.in8) CK = std::max(32, CK);
-            // untuned: TMA-store epilogue where it fits next to two pipeline stages
+            int E = 8;
+            if (!tc_variant_forced() && halo_pick(L, ty.in8 ? 1 : 2, CK, B, W, H, g_num_sms, R, P, E) &&
+                tc_conv_halo(L, src0, src1, out, pool_out, head_wh, head_bh, head_out, B, W, H, head_o, R, P, CK, 0, E, st,
+                             ty))
+                return;
+            // a forced variant (tests): TMA-store epilogue where it fits next to two pipeline stages
             // LNR_CONV_TMA_STORE=0: direct stores; =1: one staging buffer per warp
             static const int tma_store = [] {
                 const char* e = getenv("LNR_CONV_TMA_STORE");

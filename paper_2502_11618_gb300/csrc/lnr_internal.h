@@ -276,6 +276,7 @@ std::vector<TcConfig> tc_candidates(const ConvLayer& L, lnr_precision p);
 bool tc_fused_enc0(const ConvLayer& L0, const ConvLayer& L1, lnr_precision p, const void* in, void* out,
                    void* pool_out, int B, int W, int H, int R, cudaStream_t st);
 cudaError_t tc_prepare_fp8(ConvLayer& L);
+bool tc_variant_forced();  // an LNR_CONV_* switch of the tests asks for one kernel variant
 int tc_error_word();  // nonzero after a bounded wait in a tensor-core kernel ran out (then reset)
 
 }  // namespace lnr

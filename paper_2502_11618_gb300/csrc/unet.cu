@@ -264,19 +264,26 @@ static void run_call(const Unet& u, const ConvCall& k, Workspace& ws, lnr_precis
                 u.out_ch, st, force);
 }
 
-// Rows per tile of the fused level-0 encoder for the layer resolution (W, H), or 0 to run
-// the first two convs apart: the autotuner's choice, else LNR_CONV_FUSE0=2|4 (tests).
-static int fuse_rows(const Unet& u, lnr_precision p, int W, int H) {
+// Rows per tile of the fused level-0 encoder for B images at the layer resolution (W, H), or
+// 0 to run the first two convs apart: the autotuner's choice, else LNR_CONV_FUSE0=0|2|4
+// (tests), else 4 rows where its tiles (4 rows x 126 columns) number at least 300, about two
+// for every SM of the chip.  There it beats the two convs apart (one view: 1920x1080 77
+// against 111 us, 640x360 19 against 27; same results bit for bit); a 256x256 view has 192
+// tiles in two uneven waves and a third of its columns idle: it takes 152 CTAs for 12.6 us
+// where the convs apart take 64 CTAs for 19, which frames sharing the GPU pay for.
+static int fuse_rows(const Unet& u, lnr_precision p, int B, int W, int H) {
     if (p == LNR_FP32 || u.convs.size() < 2) return 0;
     static const int forced = [] {
         const char* e = getenv("LNR_CONV_FUSE0");
-        const int v = e ? atoi(e) : 0;
-        return v == 2 || v == 4 ? v : 0;
+        const int v = e ? atoi(e) : -1;
+        return v == 0 || v == 2 || v == 4 ? v : -1;
     }();
     const auto& table = p == LNR_FP8 ? u.convs[0].tuned8 : u.convs[0].tuned;
     auto it = table.find({W, H});
     if (it != table.end() && it->second.F) return it->second.F;
-    return forced;
+    if (forced >= 0) return forced;
+    if (it != table.end() || tc_variant_forced()) return 0;
+    return (int64_t)B * ((H + 3) / 4) * ((W + 125) / 126) >= 300 ? 4 : 0;
 }
 
 void unet_forward(const lnr_ctx* c, Workspace& ws, lnr_precision p, const void* in, float* out,
@@ -289,7 +296,7 @@ void unet_forward(const lnr_ctx* c, Workspace& ws, lnr_precision p, const void* 
     for (size_t i = 0; i < calls.size(); ++i) {
         const ConvCall& k = calls[i];
         if (k.layer == 0 && i + 1 < calls.size() && ws.allow_fuse) {
-            const int R = fuse_rows(u, p, k.W, k.H);
+            const int R = fuse_rows(u, p, ws.B, k.W, k.H);
             const ConvCall& k1 = calls[i + 1];
             if (R && tc_fused_enc0(u.convs[0], u.convs[1], p, k.src0, k1.out, k1.pool, ws.B, k.W, k.H, R, st)) {
                 ++i;  // both convs done
