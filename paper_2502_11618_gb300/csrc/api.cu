@@ -336,7 +336,7 @@ static lnr_status finish_output(lnr_ctx* c, Workspace& ws, float* out, size_t nf
         if (e != cudaSuccess) return cuda_fail(c, e, "render");
     }
     if (c->timing) read_timing(c, ws);
-    if ((!on_device || c->timing) && c->prec != LNR_FP32) {
+    if (!on_device || c->timing) {
         const int w = tc_error_word();
         if (w >= 5 && w <= 7) return fail(c, LNR_E_TIMEOUT, "a tensor-core kernel gave up waiting (bounded wait ran out)");
         if (w) return fail(c, LNR_E_CUDA, "a tensor-core convolution could not be launched (code " + std::to_string(w) + ")");
@@ -384,7 +384,7 @@ lnr_status lnr_destroy(lnr_ctx* c) {
     DBuf* all[] = {&c->xyz, &c->rgb, &c->scan, &c->cell_start, &c->ox, &c->oy, &c->oz, &c->rgbs};
     for (DBuf* b : all) b->release();
     for (auto& L : c->unet.convs) {
-        if (L.w32) cudaFree(L.w32);
+        if (L.wsplit) cudaFree(L.wsplit);
         if (L.b32) cudaFree(L.b32);
         if (L.wtc) cudaFree(L.wtc);
         for (void* w : L.wh)
@@ -529,11 +529,9 @@ lnr_status lnr_shard_finish(lnr_ctx* c, const lnr_view* view, const lnr_intrinsi
     if (!e) e = cudaStreamSynchronize(ws.stream);
     if (!e) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "shard_finish");
-    if (c->prec != LNR_FP32) {
-        const int w = tc_error_word();
-        if (w >= 5 && w <= 7) return fail(c, LNR_E_TIMEOUT, "a tensor-core kernel gave up waiting (bounded wait ran out)");
-        if (w) return fail(c, LNR_E_CUDA, "a tensor-core convolution could not be launched (code " + std::to_string(w) + ")");
-    }
+    const int w = tc_error_word();
+    if (w >= 5 && w <= 7) return fail(c, LNR_E_TIMEOUT, "a tensor-core kernel gave up waiting (bounded wait ran out)");
+    if (w) return fail(c, LNR_E_CUDA, "a tensor-core convolution could not be launched (code " + std::to_string(w) + ")");
     return LNR_OK;
 }
 
@@ -577,7 +575,7 @@ lnr_status lnr_set_unet(lnr_ctx* c, const lnr_unet_desc* d, const float* w, size
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
     for (auto& Lr : c->unet.convs) {
-        if (Lr.w32) cudaFree(Lr.w32);
+        if (Lr.wsplit) cudaFree(Lr.wsplit);
         if (Lr.b32) cudaFree(Lr.b32);
         if (Lr.wtc) cudaFree(Lr.wtc);
         for (void* w : Lr.wh)
@@ -831,7 +829,7 @@ lnr_status lnr_autotune(lnr_ctx* c, int W, int H, int batch) {
     const void* out_before = ws.out.p;
     if (!e) e = ws.act[4 * kMaxUnetLevels].ensure((size_t)batch * W * H * unet_in_bytes_per_px(c->prec) + 256);
     if (!e) e = ws.out.ensure((size_t)batch * W * H * 12);
-    if (!e) e = unet_ensure(c->unet, ws, LNR_FP32);
+    if (!e) e = unet_ensure(c->unet, ws, c->prec);
     if (e != cudaSuccess) return cuda_fail(c, e, "autotune buffers");
     if (in_before != ws.act[4 * kMaxUnetLevels].p || out_before != ws.out.p) ws.alloc_gen++;
     return unet_autotune(c, ws, c->prec, 3);

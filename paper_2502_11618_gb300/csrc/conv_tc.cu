@@ -23,16 +23,13 @@
 //  warps 2-5 epilogue: tcgen05.ld, bias, ReLU, BF16 store (+ pool / head).
 // Every mbarrier wait is bounded (about 2 s); a wait that runs out sets an error word and
 // the CTA drains its copies, frees its TMEM and exits.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-#include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
 #include <cstdlib>
 #include <type_traits>
 #include <cstring>
 
-#include "lnr_internal.h"
+#include "tc_ptx.h"
 
 namespace lnr {
 namespace {
@@ -43,7 +40,6 @@ constexpr int kThreads = 192;
 // between two issuers), then EPI epilogue warps.  Each issuer owns disjoint accumulators.
 // An issuing thread shares its scheduler with the epilogue warps of its TMEM lane quarter,
 // so small-N convolutions, whose MMAs are short, are issued from several threads.
-constexpr int kMmaWarps = 4;
 __host__ __device__ constexpr int halo_mma_warps(int par, int r) {
     return par == 0 ? 2 : ((par == 4 ? 2 : 1) * r < kMmaWarps ? (par == 4 ? 2 : 1) * r : kMmaWarps);
 }
@@ -52,7 +48,6 @@ __host__ __device__ constexpr int halo_mma_warps(int par, int r) {
 // 128 registers per thread).  12 for standard tiles and for tiles of two parity classes and
 // at most two rows, whose two issuers leave room for them.
 __host__ __device__ constexpr int halo_threads(int par, int r, int epi) { return 32 * (1 + halo_mma_warps(par, r) + epi); }
-constexpr long long kWaitCycles = 4000000000ll;  // ~2 s at 2 GHz
 constexpr long long kStallWaitCycles = 2000000ll;  // ~1 ms: the timeout test's wait
 constexpr int kXchStride = 33;                   // floats per row of the pooling exchange
 
@@ -85,112 +80,6 @@ struct Params {
     int head_o;
     int* err;
 };
-
-// ------------------------------------------------------------- PTX wrappers ----
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// One bounded try: the thread may sleep in the barrier until the phase completes, for at
-// most the suspend-time hint (10 ms), instead of spinning and taking issue slots from the
-// epilogue warps of its scheduler.
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(10000000u)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait for the phase of parity `parity`: false after `limit` cycles (~2 s by default).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long limit = kWaitCycles) {
-    if (mbar_try(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try(bar, parity))
-        if (clock64() - t0 > limit) return false;
-    return true;
-}
-
-__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"((uint64_t)m), "r"(c0), "r"(c1), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tma_4d(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2, int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-        "l"((uint64_t)m), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2, int c3,
-                                       int c4) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
-        "l"((uint64_t)m), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
-        : "memory");
-}
-
-__device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(ncols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-__device__ __forceinline__ void mma_fp8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-template <bool IN8>
-__device__ __forceinline__ void mma_op(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    if (IN8) mma_fp8(d, a, b, idesc, acc);
-    else mma_bf16(d, a, b, idesc, acc);
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// 16 consecutive FP32 columns of this warp's 32 TMEM lanes (one lane per thread).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
-}
-
-// UMMA shared-memory descriptor of a K-major, swizzled operand tile.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t sbo, uint32_t swz) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(sbo >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)swz << 61);
-}
-
-__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 struct TileCoord {
     int n, x0, y0;    // standard tiles: image, first column, first row
@@ -431,7 +320,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tc(const __grid_constant__
 // double-buffered).  2x2 pooling needs no shared-memory exchange: a thread owns one column
 // of R rows and its horizontal neighbour is the adjacent lane.
 
-constexpr int kHaloW = 130;  // staged pixels per halo row
 constexpr int kHaloMaxN = 256;  // output channels of one halo-kernel launch, at most
 
 struct HSeg {
@@ -492,13 +380,6 @@ struct HParams {
     alignas(16) float chead[4 * kHaloMaxN + 4];
 };
 
-__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"((uint64_t)m), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
-        : "memory");
-}
-
 // 16 channels of one pixel as E4M3 of v * inv (16 bytes, saturating).
 __device__ __forceinline__ void st_fp8x16(uint8_t* dst, const float* v, float inv) {
     uint4 pk;
@@ -507,13 +388,6 @@ __device__ __forceinline__ void st_fp8x16(uint8_t* dst, const float* v, float in
     for (int j = 0; j < 8; ++j)
         ph[j] = __nv_cvt_float2_to_fp8x2(make_float2(v[2 * j] * inv, v[2 * j + 1] * inv), __NV_SATFINITE, __NV_E4M3);
     *reinterpret_cast<uint4*>(dst) = pk;
-}
-
-// 32 bytes to a 32-byte-aligned global address in one store.
-__device__ __forceinline__ void st_32b(void* dst, uint4 a, uint4 b) {
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(a.x), "r"(a.y), "r"(a.z),
-                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
-                 : "memory");
 }
 
 // ReLU of 16 values, rounded to BF16 and packed two per word (lower half the even element).
@@ -595,172 +469,6 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 __device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 // every committed store is complete
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
-// 16 TMEM columns of this warp's lanes into r without waiting; tmem_wait16 completes it.
-__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-// Waits for every TMEM load this thread issued; r is threaded through so that no use of
-// it can be scheduled before the wait.
-__device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-                 :
-                 : "memory");
-}
-
-// High bits of a swizzled K-major UMMA descriptor (everything but the start address).
-__device__ __forceinline__ uint64_t sdesc_hi(uint32_t sbo, uint32_t swz) {
-    return ((uint64_t)1 << 16) | ((uint64_t)(sbo >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)swz << 61);
-}
-
-// ---- MMA issue of one pipeline stage, fully unrolled ----
-//
-// One thread issues about one tcgen05.mma per 50-110 cycles; loop control and descriptor
-// arithmetic with run-time bounds made that several times slower.  The issue sequence of a
-// stage is therefore unrolled at compile time over taps, K steps (NK MMAs of 32 bytes of
-// K) and the issuer's rows / units, so that every descriptor is a per-stage base plus a
-// constant.
-
-// Work split of a tile among its MMA-issuing threads: standard tiles give each of
-// issuers(R) threads RPI consecutive output rows; parity tiles give each of up to four
-// threads UPI (row, y class) units.
-template <int R, int PAR>
-struct IssueSplit {
-    static constexpr int NY = PAR == 4 ? 2 : 1;
-    static constexpr int units = PAR == 0 ? R : NY * R;
-    static constexpr int issuers = PAR == 0 ? (R >= 2 ? 2 : 1) : (units < kMmaWarps ? units : kMmaWarps);
-    static constexpr int per = units / issuers;
-};
-
-struct IssueCtx {
-    int g;           // issuer index
-    int px, py;      // parity class of the tile (PAR 1 and 2)
-    uint32_t N;      // output channels
-    uint32_t idesc;  // instruction descriptor for N columns
-};
-
-__device__ __forceinline__ uint32_t idesc_n(uint32_t idesc, uint32_t n) {
-    return (idesc & ~(0x3Fu << 17)) | ((n >> 3) << 17);
-}
-
-template <int R, int PAR, bool IN8, int NK>
-__device__ __forceinline__ void issue_stage(const IssueCtx& q, int sg, uint32_t a0, uint32_t b0, const HSeg& s, uint32_t d0,
-                                            bool first) {
-    using Sp = IssueSplit<R, PAR>;
-    constexpr int PER = Sp::per;
-    const uint32_t N = q.N;
-    const uint32_t pitch16 = s.pitch >> 4, row16 = kHaloW * pitch16, btap = N * pitch16;
-    const uint64_t hi = sdesc_hi(8 * s.pitch, s.swz);
-    if (PAR == 0) {
-        // Halo row h shifted by kx feeds output rows r = h - ky, ky = 0..2; the rows of one
-        // halo row go into one MMA (accumulators adjacent in TMEM, weight blocks [kx][ky =
-        // 2,1,0] adjacent in shared memory, N = rows * Cout <= 256).  In the stage's first
-        // (kx, k) step every row is first touched alone (h = r), zeroing it on a tile's
-        // first chunk, and the rest of that step covers h - r = 1, 2.
-        const uint32_t d = d0 + (uint32_t)(q.g * PER) * N;
-        const uint32_t a = a0 + (uint32_t)(q.g * PER) * row16;
-        const uint32_t acc0 = first ? 0u : 1u;
-#pragma unroll
-        for (int kx = 0; kx < 3; ++kx)
-#pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                const uint32_t ak = a + (uint32_t)kx * pitch16 + 2 * k, bk = b0 + 2 * k;
-                if (kx == 0 && k == 0) {
-#pragma unroll
-                    for (int r = 0; r < PER; ++r)
-                        mma_op<IN8>(d + (uint32_t)r * N, hi | (uint64_t)(ak + (uint32_t)r * row16), hi | (uint64_t)(bk + 2 * btap),
-                                    q.idesc, acc0);
-#pragma unroll
-                    for (int h = 1; h < PER + 2; ++h) {
-                        const int rlo = h - 2 > 0 ? h - 2 : 0, rhi = h - 1 < PER - 1 ? h - 1 : PER - 1;
-                        const int blk = 2 - (h - rlo);
-                        mma_op<IN8>(d + (uint32_t)rlo * N, hi | (uint64_t)(ak + (uint32_t)h * row16),
-                                    hi | (uint64_t)(bk + (uint32_t)blk * btap), idesc_n(q.idesc, (uint32_t)(rhi - rlo + 1) * N), 1u);
-                    }
-                } else {
-#pragma unroll
-                    for (int h = 0; h < PER + 2; ++h) {
-                        const int rlo = h - 2 > 0 ? h - 2 : 0, rhi = h < PER - 1 ? h : PER - 1;
-                        const int blk = kx * 3 + 2 - (h - rlo);
-                        mma_op<IN8>(d + (uint32_t)rlo * N, hi | (uint64_t)(ak + (uint32_t)h * row16),
-                                    hi | (uint64_t)(bk + (uint32_t)blk * btap), idesc_n(q.idesc, (uint32_t)(rhi - rlo + 1) * N), 1u);
-                    }
-                }
-            }
-    } else {
-        constexpr int NY = Sp::NY, NX = PAR >= 2 ? 2 : 1;
-        const uint32_t plane16 = s.plane >> 4;
-        const uint32_t id2 = idesc_n(q.idesc, 2 * N);
-        const int u0 = q.g * PER;
-        if (sg == 0) {
-            // skip operand: the fine pixel of class cx at tap (ky, kx) is x-offset dxf = cx +
-            // kx - 1 from 2X, i.e. plane dxf & 1, staged column 1 + (dxf >> 1).  With both x
-            // classes in the tile, dxf = 0 and 1 serve both classes with weight blocks
-            // (ky, dxf) and (ky, dxf + 1), adjacent in shared memory, into the unit's two
-            // adjacent accumulators [cx = 1, cx = 0]: one MMA of 2N columns.
-#pragma unroll
-            for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-                for (int k = 0; k < NK; ++k)
-#pragma unroll
-                    for (int uu = 0; uu < PER; ++uu) {
-                        const int u = u0 + uu;
-                        const int r = u / NY, cy = PAR == 4 ? u - r * NY : q.py;
-                        const uint32_t du = d0 + (uint32_t)(u * NX) * N;
-                        const uint32_t ar = a0 + (uint32_t)((PAR == 4 ? cy : 0) + ky + 2 * r) * row16 + 2 * k;
-                        auto A = [&](int dxf) {
-                            return hi | (uint64_t)(ar + (uint32_t)(dxf & 1) * plane16 + (uint32_t)(1 + (dxf >> 1)) * pitch16);
-                        };
-                        const uint32_t bk = b0 + (uint32_t)(3 * ky) * btap + 2 * k;
-                        const uint32_t init = (first && ky == 0 && k == 0) ? 0u : 1u;
-                        if (NX == 2) {
-                            mma_op<IN8>(du, A(0), hi | (uint64_t)bk, id2, init);
-                            mma_op<IN8>(du, A(1), hi | (uint64_t)(bk + btap), id2, 1u);
-                            mma_op<IN8>(du + N, A(-1), hi | (uint64_t)bk, q.idesc, 1u);
-                            mma_op<IN8>(du, A(2), hi | (uint64_t)(bk + 2 * btap), q.idesc, 1u);
-                        } else {
-                            mma_op<IN8>(du, A(q.px - 1), hi | (uint64_t)bk, q.idesc, init);
-                            mma_op<IN8>(du, A(q.px), hi | (uint64_t)(bk + btap), q.idesc, 1u);
-                            mma_op<IN8>(du, A(q.px + 1), hi | (uint64_t)(bk + 2 * btap), q.idesc, 1u);
-                        }
-                    }
-        } else {
-            // nearest-upsampled operand: class (cx, cy) reads coarse rows cy - 1 + j (j = 0,
-            // 1) and columns dxc in {cx - 1, cx}, each with the sum of the 3x3 taps that land
-            // on that coarse pixel (blocks per (cy, j): [cx=1 dxc=+1][cx=1 dxc=0][cx=0 dxc=0]
-            // [cx=0 dxc=-1]); dxc = 0 serves both x classes with one MMA of 2N columns.
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int k = 0; k < NK; ++k)
-#pragma unroll
-                    for (int uu = 0; uu < PER; ++uu) {
-                        const int u = u0 + uu;
-                        const int r = u / NY, cy = PAR == 4 ? u - r * NY : q.py;
-                        const uint32_t du = d0 + (uint32_t)(u * NX) * N;
-                        const uint32_t ar = a0 + (uint32_t)(r + cy + j) * row16 + 2 * k;
-                        const uint32_t bj = b0 + (uint32_t)((PAR == 4 ? 8 * cy : 0) + 4 * j) * btap + 2 * k;
-                        if (NX == 2) {
-                            mma_op<IN8>(du, hi | (uint64_t)(ar + 2 * pitch16), hi | (uint64_t)bj, q.idesc, 1u);
-                            mma_op<IN8>(du, hi | (uint64_t)(ar + pitch16), hi | (uint64_t)(bj + btap), id2, 1u);
-                            mma_op<IN8>(du + N, hi | (uint64_t)ar, hi | (uint64_t)(bj + 3 * btap), q.idesc, 1u);
-                        } else {
-                            // one class: cx = 1 uses blocks 0, 1 at columns +1, 0; cx = 0 blocks 2, 3 at 0, -1
-                            const uint32_t c1 = q.px ? 2 * pitch16 : pitch16;
-                            const uint32_t bb = bj + (q.px ? 0u : 2 * btap);
-                            mma_op<IN8>(du, hi | (uint64_t)(ar + c1), hi | (uint64_t)bb, q.idesc, 1u);
-                            mma_op<IN8>(du, hi | (uint64_t)(ar + c1 - pitch16), hi | (uint64_t)(bb + btap), q.idesc, 1u);
-                        }
-                    }
-        }
-    }
-}
 
 // PAR = 0: standard tiles of R rows x 128 columns.  PAR = 1, 2 or 4: the decoder's first
 // conv; a tile is R coarse rows x 128 coarse columns and PAR of the four parity classes
@@ -893,6 +601,7 @@ __global__ void __launch_bounds__(halo_threads(PAR, R, EPI), 1) k_conv_halo(cons
             const uint32_t d0 = tmem + (uint32_t)(b * NACC * N);
             for (int sg = 0; sg < p.nseg && ok; ++sg) {
                 const HSeg& s = p.seg[sg];
+                const StageGeom geo{s.pitch, s.plane, s.swz};
                 const int nk = (int)(s.pitch >> 5);  // one MMA per 32 bytes of K (16 BF16 or 32 E4M3)
                 for (int cc = 0; cc < s.nchunk; ++cc) {
                     if (!mbar_wait(full(st), ph)) { ok = false; break; }
@@ -900,9 +609,9 @@ __global__ void __launch_bounds__(halo_threads(PAR, R, EPI), 1) k_conv_halo(cons
                     const uint32_t a0 = (base + st * p.stage_bytes) >> 4;
                     const uint32_t b0 = a0 + (s.b_off >> 4);
                     switch (nk) {
-                        case 1: issue_stage<R, PAR, IN8, 1>(q, sg, a0, b0, s, d0, cc == 0); break;
-                        case 2: issue_stage<R, PAR, IN8, 2>(q, sg, a0, b0, s, d0, cc == 0); break;
-                        default: issue_stage<R, PAR, IN8, 4>(q, sg, a0, b0, s, d0, cc == 0); break;
+                        case 1: issue_stage<R, PAR, IN8, 1>(q, sg, a0, b0, geo, d0, sg == 0 && cc == 0); break;
+                        case 2: issue_stage<R, PAR, IN8, 2>(q, sg, a0, b0, geo, d0, sg == 0 && cc == 0); break;
+                        default: issue_stage<R, PAR, IN8, 4>(q, sg, a0, b0, geo, d0, sg == 0 && cc == 0); break;
                     }
                     issued = true;
                     mma_commit(empty(st));
@@ -1394,13 +1103,8 @@ __global__ void __launch_bounds__(kFuseThreads, 1) k_enc0_fused(const __grid_con
         // A(k) for the k-th tile of this CTA as soon as the first epilogue has read A(k-1);
         // then B(k-1) once its activations are in shared memory.
         IssueCtx qa{warp - 1, 0, 0, (uint32_t)N1, p.idesc1}, qb{warp - 1, 0, 0, (uint32_t)N2, p.idesc2};
-        HSeg h1, h2;
-        h1.pitch = 32;  // the 16-channel input
-        h1.swz = 6;
-        h1.plane = 0;
-        h2.pitch = p.pitch1;
-        h2.swz = p.swz1;
-        h2.plane = 0;
+        const StageGeom h1{32, 0, 6};  // the 16-channel input
+        const StageGeom h2{p.pitch1, 0, p.swz1};
         bool ok = mbar_wait(wbar, 0);
         int st = 0;
         uint32_t ph = 0u;
@@ -1548,34 +1252,12 @@ __global__ void __launch_bounds__(kFuseThreads, 1) k_enc0_fused(const __grid_con
 
 // ------------------------------------------------------------------ host side ----
 
-// cuTensorMapEncodeTiled through the runtime's driver entry-point lookup, so that the
-// library links no driver library and loads on machines without one.
-static CUresult encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, void* addr, const cuuint64_t* dims,
-                             const cuuint64_t* strides, const cuuint32_t* box, const cuuint32_t* es,
-                             CUtensorMapInterleave il, CUtensorMapSwizzle sw, CUtensorMapL2promotion l2,
-                             CUtensorMapFloatOOBfill oob) {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            f = nullptr;
-        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-    }();
-    if (!fn) return CUDA_ERROR_NOT_SUPPORTED;
-    return fn(m, dt, rank, addr, dims, strides, box, es, il, sw, l2, oob);
-}
-
 // Chunk width of a K segment of C channels (C a multiple of 16): the largest of 64, 32, 16
 // that is at most ckmax and divides C.
 int seg_ck(int C, int ckmax) {
     int ck = std::min(C, ckmax);
     while (C % ck) ck >>= 1;
     return ck;
-}
-
-CUtensorMapSwizzle swizzle_pitch(uint32_t pitch) {
-    return pitch == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : pitch == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
 }
 
 CUtensorMapSwizzle swizzle_for(int kc) {
@@ -1722,7 +1404,6 @@ static void tc_conv_generic(const ConvLayer& L, const void* src0, const void* sr
 
 // ---- halo kernel host side ----
 
-static uint32_t align_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 static int ck_index(int ck) { return ck == 16 ? 0 : ck == 32 ? 1 : 2; }
 
 
@@ -1736,7 +1417,7 @@ static int ck_index(int ck) { return ck == 16 ? 0 : ck == 32 ? 1 : 2; }
 //    the conv of the upsampled tensor is a 2x2 conv of the coarse one with summed taps.
 //    Blocks per (cy, j = coarse row cy - 1 + j): [cx=1 dxc=+1][cx=1 dxc=0][cx=0 dxc=0]
 //    [cx=0 dxc=-1], 16 per chunk.
-static std::vector<uint16_t> halo_blocks(const ConvLayer& L, int sg) {
+std::vector<uint16_t> halo_blocks(const ConvLayer& L, int sg) {
     std::vector<uint16_t> b;
     if (!L.cin1) {
         for (int j = 0; j < 9; ++j) b.push_back((uint16_t)(1u << ((2 - j % 3) * 3 + j / 3)));
@@ -2453,6 +2134,18 @@ std::vector<TcConfig> tc_candidates(const ConvLayer& L, lnr_precision prec) {
         }
     return out;
 }
+
+int* tc_err_ptr() {
+    tc_init();
+    return g_err;
+}
+
+int tc_num_sms() {
+    tc_init();
+    return g_num_sms;
+}
+
+void tc_host_error(int code) { g_host_err = code; }
 
 int tc_error_word() {
     if (g_host_err) {

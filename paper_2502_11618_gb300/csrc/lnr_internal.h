@@ -29,6 +29,19 @@ constexpr int kMaxUnetLevels = 8;
 inline thread_local uint64_t tl_launches = 0;
 inline void count_launch() { ++tl_launches; }
 
+// An FP32 value's leading part in the three-part BF16 form of the FP32 network (conv_split.cu):
+// v rounded to kHiBits significant bits, halves away from zero.  Finite values whose rounding
+// would overflow are cut instead.
+constexpr int kHiBits = 7;
+__host__ __device__ inline float split_hi(float v) {
+    constexpr uint32_t drop = 24 - kHiBits;
+    union { float f; uint32_t u; } a, b;
+    a.f = v;
+    b.u = (a.u + (1u << (drop - 1))) & ~((1u << drop) - 1);
+    if ((b.u & 0x7f800000u) == 0x7f800000u) b.u = a.u & ~((1u << drop) - 1);
+    return b.f;
+}
+
 // Parameters of one view on the device (filled by the host in FP64, then rounded once).
 struct ViewDev {
     int32_t anchor[3];
@@ -54,12 +67,11 @@ struct TcConfig {
 struct ConvLayer {
     int cin0 = 0;       // channels read from the same-resolution source
     int cin1 = 0;       // channels read from the half-resolution source (nearest 2x up)
-    int cin_pad = 0;    // cin0 + cin1 rounded up to the kernel's K granularity
     int cout = 0;
     int level = 0;
     bool pool = false;  // also write the 2x2 max-pooled output (encoder convs below the bottom)
     bool head = false;  // fuse the 1x1 head + sigmoid (last decoder conv)
-    float* w32 = nullptr;   // device, FP32 [tap][cin_pad][cout]
+    void* wsplit = nullptr; // device, FP32 weights in three BF16 parts (conv_split.cu)
     float* b32 = nullptr;   // device, FP32 [cout]
     void* wtc = nullptr;    // device, tensor-core weights [cout][tap][cin_pad] (bf16 or fp8)
     void* wh[3] = {nullptr, nullptr, nullptr};  // device, halo-kernel weights for chunks of <= 16 / 32 / 64 channels
@@ -236,7 +248,8 @@ size_t splat_max_chunks(uint64_t npoints);  // entries per view of the splat's c
 void launch_training_input(const Workspace& ws, const float* gt, float zfar, int unfiltered, float* out,
                            cudaStream_t st);
 // Upsample step from level l+1 to level l; at l == 0 also packs the U-Net input.
-// unet_in_kind: 0 = FP32 NHWC8, 1 = BF16 NHWC16, 2 = none (stage taps only).
+// unet_in_kind: 0 = FP32 NHWC8 (stage taps), 1 = BF16 NHWC16, 2 = none, 3 = FP32 as three BF16
+// parts, NHWC16 hi5 | mid5 | lo5 | 0 (the FP32 network).
 void launch_upsample(const lnr_ctx* c, Workspace& ws, int l, void* unet_in, int unet_in_kind,
                      bool write_u0, cudaStream_t st);
 size_t pyramid_floats(int W, int H, int nlev);
@@ -276,7 +289,20 @@ std::vector<TcConfig> tc_candidates(const ConvLayer& L, lnr_precision p);
 bool tc_fused_enc0(const ConvLayer& L0, const ConvLayer& L1, lnr_precision p, const void* in, void* out,
                    void* pool_out, int B, int W, int H, int R, cudaStream_t st);
 cudaError_t tc_prepare_fp8(ConvLayer& L);
+std::vector<uint16_t> halo_blocks(const ConvLayer& L, int sg);  // weight blocks of a K segment, as tap masks
+int* tc_err_ptr();             // device error word of the bounded waits
+int tc_num_sms();
+void tc_host_error(int code);  // a launch that failed on the host: the next tc_error_word reports it
 bool tc_variant_forced();  // an LNR_CONV_* switch of the tests asks for one kernel variant
+
+// conv_split.cu: the FP32 network's convolutions.  Sources and outputs are [image][hi, mid,
+// lo][C / 16][H][W][16] BF16, the first conv's source the 16-channel input.  logits (the last
+// conv, instead of out): its channels' shares of the 1x1 head's sums, [image][head
+// part][4][H][W] FP32.
+cudaError_t split_prepare_layer(ConvLayer& L);
+int split_head_parts(const ConvLayer& L);
+void conv_split(const ConvLayer& L, const void* src0, const void* src1, void* out, void* pool_out, float* logits,
+                const float* head_wh, int head_o, int B, int W, int H, cudaStream_t st);
 int tc_error_word();  // nonzero after a bounded wait in a tensor-core kernel ran out (then reset)
 
 }  // namespace lnr

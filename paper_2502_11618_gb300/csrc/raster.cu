@@ -442,8 +442,8 @@ struct UpArgs {
     int fill;            // non-final level: fill empty pixels by interpolation
     // final level only
     const uint32_t* rgba;
-    void* unet_in;       // NHWC: 8 FP32 channels (kind 0) or 16 BF16 channels (kind 1)
-    int kind;            // 0 = FP32, 1 = BF16, 2 = none
+    void* unet_in;       // NHWC network input, by the kernels' KIND: 0 = 8 FP32 channels, 1 = 16 BF16
+                         // channels, 2 = none, 3 = FP32 as 16 BF16 channels hi5 | mid5 | lo5 | 0
     float* u0;           // kept depth tap (nullable)
 };
 
@@ -455,37 +455,57 @@ __device__ __forceinline__ void st_sector(void* dst, uint32_t w0, uint32_t w1, u
                  : "memory");
 }
 
-// One pixel of the network input: 8 FP32 channels or 16 BF16 channels (32 bytes in both
-// layouts), written as one sector.
-__device__ __forceinline__ void store_unet_in(void* base, int kind, size_t q, float r, float g, float b,
-                                              float d, float a) {
-    if (kind == 0) {
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// One pixel of the network input: 8 FP32 channels or 16 BF16 channels (32 bytes in every
+// layout), written as one sector.
+template <int KIND>
+__device__ __forceinline__ void store_unet_in(void* base, size_t q, float r, float g, float b, float d, float a) {
+    if (KIND == 0) {
         st_sector(static_cast<float*>(base) + q * 8, __float_as_uint(r), __float_as_uint(g), __float_as_uint(b),
                   __float_as_uint(d), __float_as_uint(a), 0u, 0u, 0u);
-    } else if (kind == 1) {
+    } else if (KIND == 1) {
         __nv_bfloat162 v0 = __floats2bfloat162_rn(r, g), v1 = __floats2bfloat162_rn(b, d);
         __nv_bfloat162 v2 = __floats2bfloat162_rn(a, 0.f);
         st_sector(static_cast<uint4*>(base) + 2 * q, *reinterpret_cast<uint32_t*>(&v0), *reinterpret_cast<uint32_t*>(&v1),
                   *reinterpret_cast<uint32_t*>(&v2), 0u, 0u, 0u, 0u, 0u);
+    } else if (KIND == 3) {
+        const float v[5] = {r, g, b, d, a};
+        float h[5], m[5], l[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            h[i] = split_hi(v[i]);
+            const float rest = __fsub_rn(v[i], h[i]);
+            m[i] = __bfloat162float(__float2bfloat16_rn(rest));
+            l[i] = __fsub_rn(rest, m[i]);
+        }
+        st_sector(static_cast<uint4*>(base) + 2 * q, bf16_pair(h[0], h[1]), bf16_pair(h[2], h[3]), bf16_pair(h[4], m[0]),
+                  bf16_pair(m[1], m[2]), bf16_pair(m[3], m[4]), bf16_pair(l[0], l[1]), bf16_pair(l[2], l[3]),
+                  bf16_pair(l[4], 0.f));
     }
 }
 
+template <int KIND>
 __device__ __forceinline__ void pack_pixel(const UpArgs& a, const ViewDev& v, int view, size_t q, bool keep, float m) {
     const size_t P = (size_t)a.Wf * a.Hf;
     if (a.u0) a.u0[view * P + q] = keep ? m : INFINITY;
-    if (a.kind == 2) return;
+    if (KIND == 2) return;
     if (keep) {
         const uint32_t c = a.rgba[view * P + q];
-        store_unet_in(a.unet_in, a.kind, view * P + q, __fdiv_rn((float)(c & 255u), 255.0f),
+        store_unet_in<KIND>(a.unet_in, view * P + q, __fdiv_rn((float)(c & 255u), 255.0f),
                       __fdiv_rn((float)((c >> 8) & 255u), 255.0f), __fdiv_rn((float)((c >> 16) & 255u), 255.0f),
                       __fdiv_rn(m, v.zfar), 1.0f);
     } else {
-        store_unet_in(a.unet_in, a.kind, view * P + q, 0.f, 0.f, 0.f, 0.f, 0.f);
+        store_unet_in<KIND>(a.unet_in, view * P + q, 0.f, 0.f, 0.f, 0.f, 0.f);
     }
 }
 
 // One thread per coarse pixel p of a 32x8 tile; the coarse levels are staged with a
 // one-pixel clamped halo, so replicated borders come for free.
+template <int KIND>
 __global__ void __launch_bounds__(256) k_upsample(const UpArgs a) {
     __shared__ float sM[10][34], sU[10][34];
     const int view = blockIdx.z;
@@ -553,19 +573,20 @@ __global__ void __launch_bounds__(256) k_upsample(const UpArgs a) {
                 }
                 a.Uf[view * a.uf_stride + q] = val;
             } else {
-                pack_pixel(a, v, view, q, keep, m);
+                pack_pixel<KIND>(a, v, view, q, keep, m);
             }
         }
 }
 
 // n_levels = 0: no filter, every filled pixel is kept.
+template <int KIND>
 __global__ void k_pack_direct(const UpArgs a, int B) {
     const size_t P = (size_t)a.Wf * a.Hf;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < P * B; i += (size_t)gridDim.x * blockDim.x) {
         const int view = (int)(i / P);
         const size_t q = i % P;
         const float m = a.Mf[view * a.f_stride + q];
-        pack_pixel(a, a.views[view], view, q, m != INFINITY, m);
+        pack_pixel<KIND>(a, a.views[view], view, q, m != INFINITY, m);
     }
 }
 
@@ -735,7 +756,6 @@ void launch_upsample(const lnr_ctx* c, Workspace& ws, int l, void* unet_in, int 
     a.views = ws.view.as<ViewDev>();
     a.rgba = ws.rgba.as<uint32_t>();
     a.unet_in = unet_in;
-    a.kind = kind;
     a.u0 = write_u0 ? ws.u0.as<float>() : nullptr;
     int Wl = ws.W, Hl = ws.H;
     for (int k = 0; k < l; ++k) { Wl = (Wl + 1) / 2; Hl = (Hl + 1) / 2; }
@@ -744,7 +764,8 @@ void launch_upsample(const lnr_ctx* c, Workspace& ws, int l, void* unet_in, int 
     if (ws.nlev == 0) {
         a.Mf = ws.depth.as<float>();
         a.f_stride = P;
-        k_pack_direct<<<2048, 256, 0, st>>>(a, ws.B);
+        auto k = kind == 0 ? k_pack_direct<0> : kind == 1 ? k_pack_direct<1> : kind == 3 ? k_pack_direct<3> : k_pack_direct<2>;
+        k<<<2048, 256, 0, st>>>(a, ws.B);
         count_launch();
         return;
     }
@@ -756,7 +777,8 @@ void launch_upsample(const lnr_ctx* c, Workspace& ws, int l, void* unet_in, int 
     else { a.Uc = ws.pyr_u.as<float>() + pyramid_offset(ws.W, ws.H, l + 1); a.uc_stride = pstride; }
     if (l > 0) { a.Uf = ws.pyr_u.as<float>() + pyramid_offset(ws.W, ws.H, l); a.uf_stride = pstride; a.fill = 1; }
     dim3 g((a.Wc + 31) / 32, (a.Hc + 7) / 8, ws.B);
-    k_upsample<<<g, 256, 0, st>>>(a);
+    auto k = kind == 0 ? k_upsample<0> : kind == 1 ? k_upsample<1> : kind == 3 ? k_upsample<3> : k_upsample<2>;
+    k<<<g, 256, 0, st>>>(a);
     count_launch();
 }
 
@@ -907,14 +929,13 @@ extern "C" lnr_status lnr_filter_static(const float* d_depth, int W, int H, int 
     k_static_view<<<1, 1, 0, st>>>(view, S, 1.0f);
     UpArgs a{};
     a.views = view;
-    a.kind = 2;
     if (n_levels == 0) {
         a.Mf = d_depth;
         a.f_stride = (size_t)W * H;
         a.Wf = W;
         a.Hf = H;
         a.u0 = d_kept;
-        k_pack_direct<<<2048, 256, 0, st>>>(a, 1);
+        k_pack_direct<2><<<2048, 256, 0, st>>>(a, 1);
         return cudaGetLastError() == cudaSuccess ? LNR_OK : LNR_E_CUDA;
     }
     dim3 g((W + 63) / 64, (H + 63) / 64, 1);
@@ -932,7 +953,7 @@ extern "C" lnr_status lnr_filter_static(const float* d_depth, int W, int H, int 
         if (l > 0) { u.Uf = U + pyramid_offset(W, H, l); u.fill = 1; }
         else { u.Uf = nullptr; u.u0 = d_kept; u.fill = 0; }
         dim3 gu((u.Wc + 31) / 32, (u.Hc + 7) / 8, 1);
-        k_upsample<<<gu, 256, 0, st>>>(u);
+        k_upsample<2><<<gu, 256, 0, st>>>(u);
     }
     return cudaGetLastError() == cudaSuccess ? LNR_OK : LNR_E_CUDA;
 }

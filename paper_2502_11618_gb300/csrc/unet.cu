@@ -4,9 +4,10 @@
 // 1x1 head with a sigmoid.  Batch norm after the encoder convolutions is folded into them
 // when the weights are loaded.
 //
-// This file holds the FP32 path (CUDA-core implicit GEMM; the accuracy reference of the
-// GPU) and the layer orchestration shared by every precision.  Pooling, upsampling and
-// concatenation are fused into the convolutions: nothing but conv outputs is written.
+// This file holds the layer orchestration shared by every precision and the FP32 path's head.
+// Pooling, upsampling and concatenation are fused into the convolutions (conv_split.cu in
+// FP32, conv_tc.cu in BF16 and FP8): nothing but conv outputs is written.
+#include <atomic>
 #include <cmath>
 #include <cuda_bf16.h>
 #include <cstdio>
@@ -18,150 +19,21 @@
 namespace lnr {
 namespace {
 
-struct ConvArgsF32 {
-    const float* src0;  // NHWC, c0 channels, output resolution
-    const float* src1;  // NHWC, c1 channels, half resolution (read nearest-upsampled), or null
-    int c0, c1;
-    int W, H;
-    const float* w;     // [9][c0 + c1][cout]
-    const float* bias;  // [cout]
-    int cout;
-    float* out;         // NHWC, cout channels
-    float* pool_out;    // NHWC, cout channels at W/2 x H/2, or null
-};
-
-// Tile: 2 rows x TW pixels x CT output channels.  Thread = one 2x2 pixel quad x 8 output
-// channels; K is walked 8 input channels at a time, all 9 taps per chunk, from a shared
-// halo tile of 4 rows x (TW+2) pixels.
-template <int TW, int CT>
-__global__ void __launch_bounds__(256) k_conv3x3_f32(const ConvArgsF32 a) {
-    constexpr int NCOG = CT / 8;
-    constexpr int HW = TW + 2;
-    static_assert((TW / 2) * NCOG == 256, "256 threads");
-    __shared__ float sin_[8][4][HW];
-    __shared__ __align__(16) float sw[9][8][CT];
-    const int cog = threadIdx.x % NCOG, q = threadIdx.x / NCOG;
-    const int x0 = blockIdx.x * TW, y0 = blockIdx.y * 2;
-    const int nco_blocks = a.cout / CT;
-    const int view = blockIdx.z / nco_blocks;
-    const int co0 = (blockIdx.z % nco_blocks) * CT;
-    const int cin = a.c0 + a.c1;
-    const size_t P = (size_t)a.W * a.H;
-    const int Wh = a.W >> 1, Hh = a.H >> 1;
-    const float* s0 = a.src0 + view * P * a.c0;
-    const float* s1 = a.src1 ? a.src1 + view * (size_t)Wh * Hh * a.c1 : nullptr;
-    float acc[4][8];
+// End of the FP32 path's 1x1 head: out[q][o] = 1 / (1 + exp(-(b[o] + sum of the parts' sums))),
+// from the last conv's partial sums [image][part][4][pixel].  One thread per pixel.  Reading
+// the sums (24 bytes per pixel of a 32-channel net with 3 outputs) in place of the features
+// (128) took this launch on a 1080p view from 686 us, read a channel at a time, to 22 us.
+__global__ void __launch_bounds__(256) k_head_f32(const float* __restrict__ z, int parts, const float* __restrict__ b,
+                                                  int O, float* __restrict__ out, int64_t P, int64_t npx) {
+    for (int64_t q = blockIdx.x * (int64_t)256 + threadIdx.x; q < npx; q += (int64_t)gridDim.x * 256) {
+        const float* zp = z + q / P * parts * 4 * P + q % P;
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[p][j] = 0.f;
-
-    for (int cb = 0; cb < cin; cb += 8) {
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < 4 * HW * 2; idx += 256) {
-            const int h = idx & 1, j = (idx >> 1) % HW, r = (idx >> 1) / HW;
-            const int gx = x0 - 1 + j, gy = y0 - 1 + r;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (gx >= 0 && gx < a.W && gy >= 0 && gy < a.H) {
-                if (cb < a.c0)
-                    v = *reinterpret_cast<const float4*>(s0 + ((size_t)gy * a.W + gx) * a.c0 + cb + 4 * h);
-                else
-                    v = *reinterpret_cast<const float4*>(s1 + ((size_t)(gy >> 1) * Wh + (gx >> 1)) * a.c1 +
-                                                         (cb - a.c0) + 4 * h);
-            }
-            sin_[4 * h + 0][r][j] = v.x;
-            sin_[4 * h + 1][r][j] = v.y;
-            sin_[4 * h + 2][r][j] = v.z;
-            sin_[4 * h + 3][r][j] = v.w;
+        for (int o = 0; o < 4; ++o) {
+            if (o >= O) break;
+            float s = __ldg(zp + o * P);
+            for (int k = 1; k < parts; ++k) s += __ldg(zp + (4 * k + o) * P);
+            out[q * O + o] = 1.0f / (1.0f + expf(-(s + __ldg(b + o))));
         }
-        for (int idx = threadIdx.x; idx < 9 * 8 * (CT / 4); idx += 256) {
-            const int c4 = idx % (CT / 4), ci = (idx / (CT / 4)) % 8, t = idx / (CT / 4) / 8;
-            *reinterpret_cast<float4*>(&sw[t][ci][4 * c4]) =
-                *reinterpret_cast<const float4*>(a.w + ((size_t)t * cin + cb + ci) * a.cout + co0 + 4 * c4);
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int ci = 0; ci < 8; ++ci) {
-            float in[4][4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) in[r][c] = sin_[ci][r][2 * q + c];
-#pragma unroll
-            for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-                for (int kx = 0; kx < 3; ++kx) {
-                    const float4 w0 = *reinterpret_cast<const float4*>(&sw[ky * 3 + kx][ci][cog * 8]);
-                    const float4 w1 = *reinterpret_cast<const float4*>(&sw[ky * 3 + kx][ci][cog * 8 + 4]);
-                    const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-                    const float av[4] = {in[ky][kx], in[ky][kx + 1], in[ky + 1][kx], in[ky + 1][kx + 1]};
-#pragma unroll
-                    for (int p = 0; p < 4; ++p)
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) acc[p][j] = fmaf(av[p], wv[j], acc[p][j]);
-                }
-        }
-    }
-    const int co = co0 + cog * 8;
-    float b[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) b[j] = a.bias[co + j];
-    float mx[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) mx[j] = 0.f;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const int x = x0 + 2 * q + (p & 1), y = y0 + (p >> 1);
-        float o[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            o[j] = fmaxf(acc[p][j] + b[j], 0.f);
-            mx[j] = fmaxf(mx[j], o[j]);
-        }
-        if (x < a.W && y < a.H) {
-            float4* dst = reinterpret_cast<float4*>(a.out + (view * P + (size_t)y * a.W + x) * a.cout + co);
-            dst[0] = make_float4(o[0], o[1], o[2], o[3]);
-            dst[1] = make_float4(o[4], o[5], o[6], o[7]);
-        }
-    }
-    if (a.pool_out) {
-        const int px = (x0 >> 1) + q, py = y0 >> 1;
-        if (px < Wh && py < Hh) {
-            float4* dst = reinterpret_cast<float4*>(a.pool_out + (view * (size_t)Wh * Hh + (size_t)py * Wh + px) * a.cout + co);
-            dst[0] = make_float4(mx[0], mx[1], mx[2], mx[3]);
-            dst[1] = make_float4(mx[4], mx[5], mx[6], mx[7]);
-        }
-    }
-}
-
-// 1x1 head + sigmoid: out[q][o] = 1 / (1 + exp(-(b[o] + sum_c w[o][c] x[q][c]))).
-__global__ void k_head_f32(const float* __restrict__ x, int C, const float* __restrict__ w,
-                           const float* __restrict__ b, int O, float* __restrict__ out, size_t npx) {
-    size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (q >= npx) return;
-    const float* xp = x + q * C;
-    for (int o = 0; o < O; ++o) {
-        float acc = b[o];
-        for (int c = 0; c < C; ++c) acc = fmaf(w[o * C + c], xp[c], acc);
-        out[q * O + o] = 1.0f / (1.0f + expf(-acc));
-    }
-}
-
-void conv_f32(const ConvLayer& L, const float* src0, const float* src1, float* out, float* pool_out, int B,
-              int W, int H, cudaStream_t st) {
-    ConvArgsF32 a{src0, src1, L.cin0 == 5 ? 8 : L.cin0, L.cin1, W, H, L.w32, L.b32, L.cout, out, pool_out};
-    if (L.cout % 64 == 0) {
-        dim3 g((W + 63) / 64, (H + 1) / 2, B * (L.cout / 64));
-        k_conv3x3_f32<64, 64><<<g, 256, 0, st>>>(a);
-        count_launch();
-    } else if (L.cout % 32 == 0) {
-        dim3 g((W + 127) / 128, (H + 1) / 2, B * (L.cout / 32));
-        k_conv3x3_f32<128, 32><<<g, 256, 0, st>>>(a);
-        count_launch();
-    } else {
-        dim3 g((W + 255) / 256, (H + 1) / 2, B * (L.cout / 16));
-        k_conv3x3_f32<256, 16><<<g, 256, 0, st>>>(a);
-        count_launch();
     }
 }
 
@@ -170,12 +42,13 @@ inline int slot(int l, int k) { return 4 * l + k; }
 
 }  // namespace
 
-int unet_in_kind(lnr_precision p) { return p == LNR_FP32 ? 0 : 1; }
-// Bytes per pixel of the network-input buffer: 8 FP32 or 16 BF16 channels (the stage taps use
-// the FP32 layout at every precision).
+int unet_in_kind(lnr_precision p) { return p == LNR_FP32 ? 3 : 1; }
+// Bytes per pixel of the network-input buffer: 16 BF16 channels, or 8 FP32 ones (the layout
+// of the stage taps at every precision).
 size_t unet_in_bytes_per_px(lnr_precision) { return 32; }
 
-static size_t elem_bytes(lnr_precision p) { return p == LNR_FP32 ? 4 : 2; }
+// Bytes of an activation: three BF16 parts (conv_split.cu) for the FP32 network.
+static size_t elem_bytes(lnr_precision p) { return p == LNR_FP32 ? 6 : 2; }
 
 // Activation buffers of the forward pass (the network input and output are counted with the
 // frame's raster buffers): four per level, each at most the level's size (+ 256 bytes).
@@ -258,7 +131,9 @@ static void run_call(const Unet& u, const ConvCall& k, Workspace& ws, lnr_precis
                      const TcConfig* force) {
     const ConvLayer& L = u.convs[k.layer];
     if (p == LNR_FP32)
-        conv_f32(L, (const float*)k.src0, (const float*)k.src1, (float*)k.out, (float*)k.pool, ws.B, k.W, k.H, st);
+        conv_split(L, k.src0, k.src1, k.out, k.pool,
+                   k.layer + 1 == (int)u.convs.size() ? static_cast<float*>(k.out) : nullptr, u.head_wh.data(), u.out_ch,
+                   ws.B, k.W, k.H, st);
     else
         tc_conv(L, p, k.src0, k.src1, k.out, k.pool, k.head_w, k.head_b, k.head_wh, k.head_bh, k.head_out, ws.B, k.W, k.H,
                 u.out_ch, st, force);
@@ -311,8 +186,9 @@ void unet_forward(const lnr_ctx* c, Workspace& ws, lnr_precision p, const void* 
     if (p == LNR_FP32) {
         const void* deep = ws.act[slot(u.levels > 1 ? 0 : 0, u.levels > 1 ? 3 : 1)].p;
         size_t npx = (size_t)ws.B * ws.W * ws.H;
-        k_head_f32<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>((const float*)deep, u.ch[0], u.head_w, u.head_b,
-                                                                  u.out_ch, out, npx);
+        const unsigned grid = (unsigned)std::min<size_t>((npx + 255) / 256, (size_t)c->num_sms * 8);
+        k_head_f32<<<grid, 256, 0, st>>>((const float*)deep, split_head_parts(u.convs.back()), u.head_b, u.out_ch, out,
+                                         (int64_t)ws.W * ws.H, (int64_t)npx);
         count_launch();
         if (layer_ev) cudaEventRecord(layer_ev[ev++], st);
     }
@@ -521,27 +397,34 @@ lnr_status unet_autotune(lnr_ctx* c, Workspace& ws, lnr_precision p, int reps) {
 // Convert the host weights (already batch-norm folded) to the device layouts.
 lnr_status unet_prepare(lnr_ctx* c) {
     Unet& u = c->unet;
-    for (auto& L : u.convs) {
-        const int cin = L.cin0 + L.cin1;
-        const int cin_pad = (L.cin0 == 5 ? 8 : L.cin0) + L.cin1;
-        L.cin_pad = cin_pad;
-        std::vector<float> w((size_t)9 * cin_pad * L.cout, 0.f);
-        for (int co = 0; co < L.cout; ++co)
-            for (int ci = 0; ci < cin; ++ci)
-                for (int t = 0; t < 9; ++t) w[((size_t)t * cin_pad + ci) * L.cout + co] = L.wf[((size_t)co * cin + ci) * 9 + t];
-        if (L.w32) cudaFree(L.w32);
-        if (L.b32) cudaFree(L.b32);
-        if (cudaMalloc(&L.w32, w.size() * 4) || cudaMalloc(&L.b32, L.cout * 4))
-            return fail(c, LNR_E_OOM, "U-Net weight upload");
-        cudaMemcpy(L.w32, w.data(), w.size() * 4, cudaMemcpyHostToDevice);
-        cudaMemcpy(L.b32, L.bf.data(), L.cout * 4, cudaMemcpyHostToDevice);
-        if (tc_available()) {
-            for (lnr_precision p : {LNR_BF16}) {
-                cudaError_t e = tc_prepare_layer(L, p);
-                if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core weight upload");
+    // Each layer's layouts are converted on the host: up to eight threads take one at a time.
+    std::vector<cudaError_t> err(u.convs.size(), cudaSuccess);
+    std::atomic<size_t> next{0};
+    auto work = [&] {
+        cudaSetDevice(c->device);
+        for (size_t i; (i = next++) < u.convs.size();) {
+            ConvLayer& L = u.convs[i];
+            try {
+                if (L.b32) cudaFree(L.b32);
+                L.b32 = nullptr;
+                if ((err[i] = cudaMalloc(&L.b32, L.cout * 4)) != cudaSuccess) continue;
+                if ((err[i] = cudaMemcpy(L.b32, L.bf.data(), L.cout * 4, cudaMemcpyHostToDevice)) != cudaSuccess) continue;
+                if ((err[i] = split_prepare_layer(L)) != cudaSuccess) continue;
+                if (tc_available()) err[i] = tc_prepare_layer(L, LNR_BF16);
+            } catch (const std::bad_alloc&) {
+                err[i] = cudaErrorMemoryAllocation;
             }
         }
+    };
+    std::vector<std::thread> threads;
+    try {
+        while (threads.size() + 1 < std::min<size_t>(8, u.convs.size())) threads.emplace_back(work);
+    } catch (const std::exception&) {  // fewer threads, then
     }
+    work();
+    for (auto& t : threads) t.join();
+    for (cudaError_t e : err)
+        if (e != cudaSuccess) return cuda_fail(c, e, "U-Net weight upload");
     if (u.head_w) cudaFree(u.head_w);
     if (u.head_b) cudaFree(u.head_b);
     if (cudaMalloc(&u.head_w, u.head_wh.size() * 4) || cudaMalloc(&u.head_b, u.head_bh.size() * 4))
