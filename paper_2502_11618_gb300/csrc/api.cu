@@ -381,7 +381,7 @@ lnr_status lnr_destroy(lnr_ctx* c) {
     lnr_serve_stop(c);
     cudaStreamSynchronize(c->stream);
     c->ws.release();
-    DBuf* all[] = {&c->xyz, &c->rgb, &c->scan, &c->cell_start, &c->ox, &c->oy, &c->oz, &c->rgbs};
+    DBuf* all[] = {&c->xyz, &c->rgbs_in, &c->grid_tmp, &c->cell_start, &c->ox, &c->oy, &c->oz, &c->rgbs, &c->box};
     for (DBuf* b : all) b->release();
     for (auto& L : c->unet.convs) {
         if (L.wsplit) cudaFree(L.wsplit);
@@ -412,13 +412,18 @@ lnr_status lnr_load_cloud(lnr_ctx* c, const double* xyz, const uint8_t* rgb, con
         if (!std::isfinite(xyz[i])) return fail(c, LNR_E_ARG, "non-finite coordinate");
     cudaError_t e;
     c->grid_ok = false;
-    if ((e = c->xyz.ensure(24 * n)) || (e = c->rgb.ensure(3 * n)) || (scan_id && (e = c->scan.ensure(n))))
+    DBuf bytes;  // colours, then scanner ids, as they come
+    if ((e = c->xyz.ensure(24 * n)) || (e = c->rgbs_in.ensure(4 * n)) || (e = bytes.ensure((scan_id ? 4 : 3) * n)))
         return cuda_fail(c, e, "cloud upload");
-    if (!scan_id) c->scan.release();
+    uint8_t* scan = scan_id ? bytes.as<uint8_t>() + 3 * n : nullptr;
     if ((e = cudaMemcpy(c->xyz.p, xyz, 24 * n, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->rgb.p, rgb, 3 * n, cudaMemcpyHostToDevice)) ||
-        (scan_id && (e = cudaMemcpy(c->scan.p, scan_id, n, cudaMemcpyHostToDevice))))
+        (e = cudaMemcpy(bytes.p, rgb, 3 * n, cudaMemcpyHostToDevice)) ||
+        (scan_id && (e = cudaMemcpy(scan, scan_id, n, cudaMemcpyHostToDevice))) ||
+        (e = pack_rgbs(bytes.as<uint8_t>(), scan, n, c->rgbs_in.as<uint32_t>(), c->stream))) {
+        bytes.release();
         return cuda_fail(c, e, "cloud upload");
+    }
+    bytes.release();
     c->n = n;
     c->cloud_gen++;
     return LNR_OK;
@@ -458,12 +463,10 @@ lnr_status lnr_build_grid(lnr_ctx* c, double cell) {
     if (!c->n) return fail(c, LNR_E_STATE, "build_grid before load_cloud");
     if (!(cell > 0.0) || !std::isfinite(cell)) return fail(c, LNR_E_ARG, "cell size must be > 0");
     cudaSetDevice(c->device);
-    DBuf tmp;
-    cudaError_t e = tmp.ensure(1024 * 6 * sizeof(double));
+    cudaError_t e = c->box.ensure(6 * sizeof(long long));
     if (e != cudaSuccess) return cuda_fail(c, e, "grid");
     double lohi[6];
-    e = grid_bbox(c->xyz.as<double>(), c->n, tmp.as<double>(), lohi, c->stream);
-    tmp.release();
+    e = grid_bbox(c->xyz.as<double>(), c->n, c->box.as<long long>(), lohi, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "grid bounds");
     double g0[3];
     int32_t dims[3];

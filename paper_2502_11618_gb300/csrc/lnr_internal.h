@@ -195,7 +195,7 @@ struct lnr_ctx {
     std::string err;
     // cloud
     uint64_t n = 0;
-    lnr::DBuf xyz, rgb, scan;
+    lnr::DBuf xyz, rgbs_in;  // rgbs_in: r | g << 8 | b << 16 | scanner << 24 per point
     uint64_t cloud_gen = 0;
     // grid
     bool grid_ok = false;
@@ -204,6 +204,7 @@ struct lnr_ctx {
     int32_t dims[3] = {0, 0, 0};
     int64_t ncells = 0;
     lnr::DBuf cell_start, ox, oy, oz, rgbs;
+    lnr::DBuf box, grid_tmp;  // bounds of the cloud (6 words); the grid build's histograms
     // U-Net
     bool unet_ok = false;
     lnr::Unet unet;
@@ -230,8 +231,9 @@ lnr_status fail(lnr_ctx* c, lnr_status s, const std::string& msg);
 lnr_status cuda_fail(lnr_ctx* c, cudaError_t e, const char* where);
 
 // grid.cu
-cudaError_t grid_bbox(const double* xyz, uint64_t n, double* d_tmp, double out_lohi[6], cudaStream_t st);
+cudaError_t grid_bbox(const double* xyz, uint64_t n, long long* box, double out_lohi[6], cudaStream_t st);
 cudaError_t grid_build(lnr_ctx* c, cudaStream_t st);
+cudaError_t pack_rgbs(const uint8_t* rgb, const uint8_t* scan, uint64_t n, uint32_t* out, cudaStream_t st);
 
 // raster.cu
 int cull_blocks(int64_t ncells);
