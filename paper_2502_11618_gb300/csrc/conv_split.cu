@@ -119,15 +119,6 @@ __device__ __forceinline__ void st_split(__nv_bfloat16* dst, size_t part, const 
     }
 }
 
-// n contiguous bytes into shared memory.  A TMA box moves about one of its rows per cycle,
-// whatever their length: the weights' 32-byte rows would come at 25 bytes per cycle and SM
-// (measured), a contiguous copy at the L2's rate.
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t n, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(n), "r"(bar)
-                 : "memory");
-}
-
 // 8 TMEM columns of this warp's lanes; tmem_wait8 completes the load.
 __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"

@@ -127,6 +127,16 @@ __device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* m, uint3
         : "memory");
 }
 
+// n contiguous bytes into shared memory.  A TMA box moves about one of its rows per cycle,
+// whatever their length: rows of 32 bytes come at 25 bytes per cycle and SM, rows of 64 at 50
+// (measured), a contiguous copy at the L2's rate.  Weights are therefore laid out as shared
+// memory holds them, swizzle included.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t n, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(n), "r"(bar)
+                 : "memory");
+}
+
 // 32 bytes to a 32-byte-aligned global address in one store.
 __device__ __forceinline__ void st_32b(void* dst, uint4 a, uint4 b) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(a.x), "r"(a.y), "r"(a.z),
@@ -330,6 +340,13 @@ static CUresult encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t 
     }();
     if (!fn) return CUDA_ERROR_NOT_SUPPORTED;
     return fn(m, dt, rank, addr, dims, strides, box, es, il, sw, l2, oob);
+}
+
+// Byte `off` of a block of rows of `pitch` bytes (32, 64 or 128) where the TMA and UMMA swizzle
+// of that row length puts it: the 16-byte chunk index XOR address bits 7 and up.
+inline uint32_t swizzled(uint32_t off, uint32_t pitch) {
+    const uint32_t mask = pitch == 128 ? 7u : pitch == 64 ? 3u : 1u;
+    return off ^ (((off >> 7) & mask) << 4);
 }
 
 inline CUtensorMapSwizzle swizzle_pitch(uint32_t pitch) {
