@@ -123,7 +123,7 @@ static cudaError_t ensure_ws(const lnr_ctx* c, Workspace& ws, int B, int W, int 
     if ((e = ws.view.ensure(sizeof(ViewDev) * B)) || (e = ws.cull_flag.ensure(4 * c->ncells * B)) ||
         (e = ws.cull_cnt.ensure(4 * c->ncells * B)) || (e = ws.cull_bsum.ensure(8 * (size_t)nb * B)) ||
         (e = ws.vis_info.ensure(16 * c->ncells * B)) || (e = ws.vis_pref.ensure(4 * c->ncells * B)) ||
-        (e = ws.vis_tot.ensure(8 * B)) || (e = ws.chunk_cell.ensure(4 * splat_max_chunks(c->n) * B)) ||
+        (e = ws.vis_tot.ensure(8 * B)) || (e = ws.chunk_cell.ensure(4 * splat_max_chunks(c->n, B) * B)) ||
         (e = ws.depth.ensure(4 * P * B)) || (e = ws.rgba.ensure(4 * P * B)) ||
         (e = ws.pyr_m.ensure(4 * pf * B)) || (e = ws.pyr_u.ensure(4 * pf * B)) || (e = ws.u0.ensure(4 * P * B)) ||
         (e = ws.out.ensure(12 * P * B)))
@@ -253,7 +253,7 @@ size_t frame_bytes(const lnr_ctx* c, int B, int W, int H, bool soft) {
     // soft z-buffer sums 16; per view the cull and compaction tables (28 bytes per cell, block
     // sums, the splat's chunk table) and the view parameters
     const size_t per_view = 28 * (size_t)c->ncells + 8 * (size_t)cull_blocks(c->ncells) +
-                            4 * splat_max_chunks(c->n) + sizeof(ViewDev) + 8;
+                            4 * splat_max_chunks(c->n, B) + sizeof(ViewDev) + 8;
     return P * (soft ? 80 : 64) + 8 * (size_t)B * pyramid_floats(W, H, kMaxLevels) + (size_t)B * per_view + 16 * 256;
 }
 

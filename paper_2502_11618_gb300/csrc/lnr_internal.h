@@ -246,7 +246,7 @@ void launch_resolve_pyramid(const lnr_ctx* c, Workspace& ws, cudaStream_t st);
 void enqueue_from_keys(lnr_ctx* c, Workspace& ws, cudaStream_t st, const uint64_t* keys, const uint32_t* rgba,
                        int stage, lnr_precision prec);
 void launch_splat_soft(const lnr_ctx* c, Workspace& ws, cudaStream_t st);
-size_t splat_max_chunks(uint64_t npoints);  // entries per view of the splat's chunk -> first cell table
+size_t splat_max_chunks(uint64_t npoints, int nviews);  // entries per view of the splat's chunk -> first cell table
 void launch_training_input(const Workspace& ws, const float* gt, float zfar, int unfiltered, float* out,
                            cudaStream_t st);
 // Upsample step from level l+1 to level l; at l == 0 also packs the U-Net input.

@@ -26,10 +26,22 @@ namespace {
 constexpr float kEdgeRel = 0.1f;         // edge when |Laplacian| > kEdgeRel * depth
 constexpr float kCullPad = 1.0f / 64.0f; // cells grow by 1/64 of a step on every side
 constexpr int kCullThreads = 256;
-constexpr int kCullPer = 4;
-constexpr int kCullTile = kCullThreads * kCullPer;
+// Cells per thread of the cull's first pass: 1 up to 2^18 cells, where a block's serial work is
+// what takes the time (20M-point scan, 40K cells: 6.7 us with 4, 4.2 with 1), else 4, which
+// leaves the second pass fewer block sums.
+inline int cull_per(int64_t ncells) { return ncells <= (1 << 18) ? 1 : 4; }
 constexpr int kSplatThreads = 256;
-constexpr int kSplatChunk = 1024;  // visible points per splat range (one warp's unit of work)
+// Visible points per splat range (one warp's unit of work), as a power of two: 128 (one batch of
+// a warp) up to 1024, at most the visible points that every warp of the GPU would get, taking
+// a sixth of the cloud to be visible in each view.  A range of 1024 points is eight batches in a
+// row: with fewer ranges than warps the splat waits for those (200k points: 16.2 us with 1024,
+// 5.6 with 128; from 5M points on no difference), with many its cells are loaded less often.
+inline int splat_shift(uint64_t npoints, int nviews) {
+    const uint64_t per_warp = npoints * (uint64_t)nviews / (6 * 4864);  // 152 SMs x 32 warps
+    int s = 7;
+    while (s < 10 && (2ull << s) <= per_warp) ++s;
+    return s;
+}
 constexpr uint64_t kEmpty = ~0ull;
 
 __device__ __forceinline__ void cell_cam(int64_t i, int64_t j, int64_t k, const ViewDev& v, float o[3]) {
@@ -108,13 +120,14 @@ __device__ __forceinline__ void block_scan2(uint32_t a, uint32_t b, uint32_t& ea
 
 // Phase 1: visibility of every cell, block-local ranks of the visible non-empty cells and
 // of their points.  flag[c] = local rank or ~0; cnt[c] = local point prefix.
+template <int kCullPer>
 __global__ void __launch_bounds__(kCullThreads) k_cull_block(
     const ViewDev* __restrict__ views, const uint32_t* __restrict__ cell_start, int dx, int dy,
     int dz, int64_t C, int W, int H, uint32_t* __restrict__ flag, uint32_t* __restrict__ cnt,
     uint32_t* __restrict__ bsum, int nb) {
     const int view = blockIdx.y;
     const ViewDev v = views[view];
-    int64_t c0 = (int64_t)blockIdx.x * kCullTile + (int64_t)threadIdx.x * kCullPer;
+    int64_t c0 = ((int64_t)blockIdx.x * kCullThreads + threadIdx.x) * kCullPer;
     uint32_t f[kCullPer], n[kCullPer], sf = 0, sn = 0;
 #pragma unroll
     for (int e = 0; e < kCullPer; ++e) {
@@ -182,19 +195,19 @@ __global__ void __launch_bounds__(kCullThreads) k_cull_scan(uint32_t* __restrict
 // Phase 3: compaction.  For the r-th visible cell of a view: vis_info[view][r] = its
 // camera-space origin and (sorted position of its first point - visible points before it),
 // vis_pref[view][r] = visible points before it; and chunk_cell[view][k] = r for every
-// splat range k (kSplatChunk visible points) whose first point lies in this cell, so that
+// splat range k (2^shift visible points) whose first point lies in this cell, so that
 // the splat finds a range's cells without searching.
 __global__ void k_cull_compact(const ViewDev* __restrict__ views, const uint32_t* __restrict__ flag,
                                const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ bsum, int nb,
                                int64_t C, int dx, int dy, const uint32_t* __restrict__ cell_start,
                                float4* __restrict__ vis_info, uint32_t* __restrict__ vis_pref,
-                               uint32_t* __restrict__ chunk_cell, size_t max_chunks) {
+                               uint32_t* __restrict__ chunk_cell, size_t max_chunks, int shift, int cull_tile) {
     const int view = blockIdx.y;
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= C) return;
     uint32_t f = flag[(size_t)view * C + c];
     if (f == ~0u) return;
-    int b = (int)(c / kCullTile);
+    int b = (int)(c / cull_tile);
     const uint32_t* bs = bsum + ((size_t)view * nb + b) * 2;
     uint32_t r = bs[0] + f;
     const uint32_t pref = bs[1] + cnt[(size_t)view * C + c];
@@ -204,12 +217,12 @@ __global__ void k_cull_compact(const ViewDev* __restrict__ views, const uint32_t
     vis_pref[(size_t)view * C + r] = pref;
     const uint32_t n = cell_start[c + 1] - cell_start[c];  // > 0: only non-empty cells are visible
     uint32_t* cc = chunk_cell + (size_t)view * max_chunks;
-    for (uint32_t k = (pref + kSplatChunk - 1) / kSplatChunk; k <= (pref + n - 1) / kSplatChunk; ++k) cc[k] = r;
+    for (uint32_t k = (uint32_t)(((uint64_t)pref + (1u << shift) - 1) >> shift); k <= (pref + n - 1) >> shift; ++k) cc[k] = r;
 }
 
 // ------------------------------------------------------------------ splat ----
 //
-// Warps work independently (no block barriers) through ranges of kSplatChunk consecutive
+// Warps work independently (no block barriers) through ranges of 2^shift consecutive
 // visible points, the ranges of all views of the batch in one list.  For a range, lane l
 // holds visible cell (first cell of the range) + l: its camera-space origin, the offset
 // from visible-point index to sorted position and its point prefix, loaded from the
@@ -231,7 +244,7 @@ __global__ void __launch_bounds__(kSplatThreads, 4) k_splat(
     const uint32_t* __restrict__ vis_pref, const uint32_t* __restrict__ tot, const float* __restrict__ ox,
     const float* __restrict__ oy, const float* __restrict__ oz, int W, int H, unsigned long long* __restrict__ keys,
     const uint32_t* __restrict__ rgbs, unsigned long long* __restrict__ acc, float scale,
-    const uint32_t* __restrict__ chunk_cell, size_t max_chunks, uint32_t pos_base) {
+    const uint32_t* __restrict__ chunk_cell, size_t max_chunks, uint32_t pos_base, int shift) {
     __shared__ ViewDev sv[kSplatMaxViews];
     for (int i = threadIdx.x; i < nviews * (int)(sizeof(ViewDev) / 4); i += blockDim.x)
         reinterpret_cast<uint32_t*>(sv)[i] = reinterpret_cast<const uint32_t*>(views)[i];
@@ -244,11 +257,11 @@ __global__ void __launch_bounds__(kSplatThreads, 4) k_splat(
     uint64_t first = 0;  // global index of the view's first range
     for (uint64_t g = warp0;; g += nwarps) {
         // the view of global range g (ranges of view 0 first, then view 1, ...)
-        uint32_t nr = (tot[2 * view + 1] + kSplatChunk - 1) / kSplatChunk;
+        uint32_t nr = (uint32_t)(((uint64_t)tot[2 * view + 1] + (1u << shift) - 1) >> shift);
         while (g >= first + nr) {
             first += nr;
             if (++view == nviews) return;
-            nr = (tot[2 * view + 1] + kSplatChunk - 1) / kSplatChunk;
+            nr = (uint32_t)(((uint64_t)tot[2 * view + 1] + (1u << shift) - 1) >> shift);
         }
         const ViewDev& v = sv[view];
         const uint32_t nvc = tot[2 * view], npts = tot[2 * view + 1];
@@ -256,8 +269,8 @@ __global__ void __launch_bounds__(kSplatThreads, 4) k_splat(
         const uint32_t* vp = vis_pref + (size_t)view * C;
         unsigned long long* kv = keys + (size_t)view * W * H;
         const uint32_t rg = (uint32_t)(g - first);
-        const uint32_t start = rg * kSplatChunk;
-        const uint32_t end = min(start + (uint32_t)kSplatChunk, npts);
+        const uint32_t start = rg << shift;
+        const uint32_t end = npts - start < (1u << shift) ? npts : start + (1u << shift);
         uint32_t cb = chunk_cell[(size_t)view * max_chunks + rg];  // the cell holding point `start`
         for (uint32_t a = start; a < end;) {
             // lane l: visible cell cb + l
@@ -355,7 +368,8 @@ __global__ void k_fill_u64(unsigned long long* __restrict__ p, size_t n) {
 // +inf, so each level pixel is the minimum over its clipped 2^l x 2^l block).  With the
 // soft z-buffer's sums (acc non-null) the colour is their per-channel integer mean
 // (sum + n/2) / n, and the sums are reset to zero.
-__global__ void __launch_bounds__(256) k_resolve_pyramid(
+template <int T>
+__global__ void __launch_bounds__(T) k_resolve_pyramid(
     unsigned long long* __restrict__ keys, const uint32_t* __restrict__ rgbs, int W, int H, int nlev,
     float* __restrict__ depth, uint32_t* __restrict__ rgba, float* __restrict__ pyr, size_t pyr_stride,
     unsigned long long* __restrict__ acc, uint32_t pos_base, uint32_t n_local) {
@@ -369,8 +383,8 @@ __global__ void __launch_bounds__(256) k_resolve_pyramid(
     const int x = threadIdx.x & 63, y0 = threadIdx.x >> 6;
     const int gx = blockIdx.x * 64 + x;
 #pragma unroll 4
-    for (int i = 0; i < 16; ++i) {
-        const int y = y0 + 4 * i;
+    for (int i = 0; i < 4096 / T; ++i) {
+        const int y = y0 + T / 64 * i;
         const int gy = blockIdx.y * 64 + y;
         float d = INFINITY;
         if (gx < W && gy < H) {
@@ -405,12 +419,12 @@ __global__ void __launch_bounds__(256) k_resolve_pyramid(
     float* lev = pyr + view * pyr_stride;
     int Wl = W, Hl = H;
     for (int l = 1; l <= nlev; ++l) {
-        const int T = 64 >> l;                  // tile side at this level
+        const int S = 64 >> l;                  // tile side at this level
         Wl = (Wl + 1) >> 1;
         Hl = (Hl + 1) >> 1;
         // read level l-1 from s (l odd) or t (l even), write level l into the other
-        for (int idx = threadIdx.x; idx < T * T; idx += 256) {
-            const int lx = idx % T, ly = idx / T;
+        for (int idx = threadIdx.x; idx < S * S; idx += T) {
+            const int lx = idx % S, ly = idx / S;
             float m;
             if (l & 1) {
                 m = fminf(fminf(s[2 * ly][2 * lx], s[2 * ly][2 * lx + 1]),
@@ -421,7 +435,7 @@ __global__ void __launch_bounds__(256) k_resolve_pyramid(
                           fminf(t[2 * ly + 1][2 * lx], t[2 * ly + 1][2 * lx + 1]));
                 s[ly][lx] = m;
             }
-            const int ox_ = blockIdx.x * T + lx, oy_ = blockIdx.y * T + ly;
+            const int ox_ = blockIdx.x * S + lx, oy_ = blockIdx.y * S + ly;
             if (ox_ < Wl && oy_ < Hl) lev[(size_t)oy_ * Wl + ox_] = m;
         }
         lev += (size_t)Wl * Hl;
@@ -603,14 +617,18 @@ __global__ void k_extract5(const void* in, int kind, float* out, int64_t npx) {
 
 }  // namespace
 
-size_t splat_max_chunks(uint64_t npoints) { return (size_t)(npoints / kSplatChunk) + 2; }
+size_t splat_max_chunks(uint64_t npoints, int nviews) { return (size_t)(npoints >> splat_shift(npoints, nviews)) + 2; }
 
-int cull_blocks(int64_t ncells) { return (int)((ncells + kCullTile - 1) / kCullTile); }
+int cull_blocks(int64_t ncells) {
+    const int tile = kCullThreads * cull_per(ncells);
+    return (int)((ncells + tile - 1) / tile);
+}
 
 void launch_cull(const lnr_ctx* c, Workspace& ws, cudaStream_t st) {
     const int nb = cull_blocks(c->ncells);
     dim3 g1(nb, ws.B);
-    k_cull_block<<<g1, kCullThreads, 0, st>>>(ws.view.as<ViewDev>(), c->cell_start.as<uint32_t>(), c->dims[0],
+    const int per = cull_per(c->ncells);
+    (per == 1 ? k_cull_block<1> : k_cull_block<4>)<<<g1, kCullThreads, 0, st>>>(ws.view.as<ViewDev>(), c->cell_start.as<uint32_t>(), c->dims[0],
                                               c->dims[1], c->dims[2], c->ncells, ws.W, ws.H,
                                               ws.cull_flag.as<uint32_t>(), ws.cull_cnt.as<uint32_t>(),
                                               ws.cull_bsum.as<uint32_t>(), nb);
@@ -621,7 +639,8 @@ void launch_cull(const lnr_ctx* c, Workspace& ws, cudaStream_t st) {
     k_cull_compact<<<g3, 256, 0, st>>>(ws.view.as<ViewDev>(), ws.cull_flag.as<uint32_t>(), ws.cull_cnt.as<uint32_t>(),
                                        ws.cull_bsum.as<uint32_t>(), nb, c->ncells, c->dims[0], c->dims[1],
                                        c->cell_start.as<uint32_t>(), ws.vis_info.as<float4>(), ws.vis_pref.as<uint32_t>(),
-                                       ws.chunk_cell.as<uint32_t>(), splat_max_chunks(c->n));
+                                       ws.chunk_cell.as<uint32_t>(), splat_max_chunks(c->n, ws.B), splat_shift(c->n, ws.B),
+                                       kCullThreads * per);
     count_launch();
 }
 
@@ -640,7 +659,7 @@ static int splat_blocks(const lnr_ctx* c, bool soft) {
 // One launch per group of up to kSplatMaxViews views.
 template <bool SOFT>
 static void splat_views(const lnr_ctx* c, Workspace& ws, cudaStream_t st, float scale) {
-    const size_t P = (size_t)ws.W * ws.H, mc = splat_max_chunks(c->n);
+    const size_t P = (size_t)ws.W * ws.H, mc = splat_max_chunks(c->n, ws.B);
     for (int v0 = 0; v0 < ws.B; v0 += kSplatMaxViews) {
         const int nv = std::min(kSplatMaxViews, ws.B - v0);
         k_splat<SOFT><<<splat_blocks(c, SOFT), kSplatThreads, 0, st>>>(
@@ -649,7 +668,7 @@ static void splat_views(const lnr_ctx* c, Workspace& ws, cudaStream_t st, float 
             ws.vis_tot.as<uint32_t>() + 2 * v0, c->ox.as<float>(), c->oy.as<float>(), c->oz.as<float>(), ws.W, ws.H,
             ws.keys.as<unsigned long long>() + v0 * P, SOFT ? c->rgbs.as<uint32_t>() : nullptr,
             SOFT ? ws.soft_acc.as<unsigned long long>() + 2 * v0 * P : nullptr, scale,
-            ws.chunk_cell.as<uint32_t>() + (size_t)v0 * mc, mc, SOFT ? 0u : c->shard_base);
+            ws.chunk_cell.as<uint32_t>() + (size_t)v0 * mc, mc, SOFT ? 0u : c->shard_base, splat_shift(c->n, ws.B));
         count_launch();
     }
 }
@@ -739,7 +758,13 @@ size_t pyramid_floats(int W, int H, int nlev) { return pyramid_offset(W, H, nlev
 
 void launch_resolve_pyramid(const lnr_ctx* c, Workspace& ws, cudaStream_t st) {
     dim3 g((ws.W + 63) / 64, (ws.H + 63) / 64, ws.B);
-    k_resolve_pyramid<<<g, 256, 0, st>>>(ws.keys.as<unsigned long long>(), c->rgbs.as<uint32_t>(), ws.W, ws.H,
+    // 1024 threads a tile when all tiles are on the GPU at once (2 to an SM): a thread's keys and
+    // colours come one round of loads after the other, four rounds instead of sixteen (256x256
+    // 11.2 -> 5.7 us, 1080p 18.4 -> 14.4); past 8 small blocks an SM, 256 threads (eight 1080p
+    // views: 81 against 93 us)
+    const bool few = (int64_t)g.x * g.y * g.z < 8 * (int64_t)c->num_sms;
+    (few ? k_resolve_pyramid<1024> : k_resolve_pyramid<256>)<<<g, few ? 1024 : 256, 0, st>>>(
+        ws.keys.as<unsigned long long>(), c->rgbs.as<uint32_t>(), ws.W, ws.H,
                                          ws.nlev, ws.depth.as<float>(), ws.rgba.as<uint32_t>(), ws.pyr_m.as<float>(),
                                          pyramid_floats(ws.W, ws.H, ws.nlev),
                                          c->soft_rel > 0.0f ? ws.soft_acc.as<unsigned long long>() : nullptr, c->shard_base,
@@ -842,31 +867,24 @@ void launch_unet_in_extract(const void* unet_in, int kind, float* out5, int64_t 
 namespace lnr {
 namespace {
 
-// 3 Mi floats (12 MiB): one view parameter block, the min-pooled levels M1..Mn and the
-// upsampled levels U1..U(n-1).  A 2560 x 1440 image with 6 levels needs about 2.5 Mi.
+// 3 Mi floats (12 MiB): the min-pooled levels M1..Mn.  Images whose min-pooled and upsampled
+// levels together would not fit are refused (2560 x 1440 with 6 levels needs about 2.5 Mi).
 constexpr size_t kStaticFilterFloats = size_t(3) << 20;
-constexpr size_t kStaticViewFloats = 64;  // ViewDev block at the front (256-byte aligned)
-static_assert(sizeof(ViewDev) <= kStaticViewFloats * sizeof(float), "view block");
+constexpr size_t kStaticViewFloats = 64;
 
 __device__ __align__(256) float g_filter_scratch[kStaticFilterFloats];
 
-__global__ void k_static_view(ViewDev* v, float S, float zfar) {
-    ViewDev d{};
-    d.S = S;
-    d.zfar = zfar;
-    *v = d;
-}
-
 // Min-pool pyramid of a depth image, one 64 x 64 tile per block (the same levels as the
 // resolve kernel computes from z-buffer keys).
-__global__ void __launch_bounds__(256) k_pyramid_from_depth(const float* __restrict__ depth, int W, int H, int nlev,
+__global__ void __launch_bounds__(512) k_pyramid_from_depth(const float* __restrict__ depth, int W, int H, int nlev,
                                                             float* __restrict__ pyr) {
     __shared__ float s[64][65];
     __shared__ float t[32][33];
     const int x = threadIdx.x & 63, y0 = threadIdx.x >> 6;
     const int gx = blockIdx.x * 64 + x;
-    for (int i = 0; i < 16; ++i) {
-        const int y = y0 + 4 * i, gy = blockIdx.y * 64 + y;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int y = y0 + 8 * i, gy = blockIdx.y * 64 + y;
         s[y][x] = (gx < W && gy < H) ? depth[(size_t)gy * W + gx] : INFINITY;
     }
     __syncthreads();
@@ -876,7 +894,7 @@ __global__ void __launch_bounds__(256) k_pyramid_from_depth(const float* __restr
         const int T = 64 >> l;
         Wl = (Wl + 1) >> 1;
         Hl = (Hl + 1) >> 1;
-        for (int idx = threadIdx.x; idx < T * T; idx += 256) {
+        for (int idx = threadIdx.x; idx < T * T; idx += 512) {
             const int lx = idx % T, ly = idx / T;
             float m;
             if (l & 1) {
@@ -891,6 +909,128 @@ __global__ void __launch_bounds__(256) k_pyramid_from_depth(const float* __restr
         }
         lev += (size_t)Wl * Hl;
         __syncthreads();
+    }
+}
+
+// Every upsampling level of a 64 x 64 tile of the image in one block.  The block holds the
+// part of each coarse level that its tile depends on: level 1 over the tile's 32 x 32 pixels and
+// one around them, each deeper level over the pixels of the finer part and two around (34, 20,
+// 12, 8, 6, 5 pixels a side), recomputing what neighbouring tiles share (about a third of the
+// coarse work, itself a third of the fine).  Positions outside the image hold the values of the
+// nearest pixel inside, as the replicated borders of the method.  One launch in place of one
+// per level, whose grids of a few blocks each took 5 us one after the other: 1920x1080 with 5
+// levels, whole call 39.9 -> 24.4 us.
+struct FusedLevel {
+    int W, H;        // level size
+    const float* M;  // min-pooled level
+};
+struct FusedArgs {
+    FusedLevel lev[kMaxLevels + 1];  // [1..n]
+    const float* depth;
+    float* kept;
+    int W, H, n;
+    float S;
+};
+__host__ __device__ constexpr int fused_side(int l) { return l == 1 ? 34 : l == 2 ? 20 : l == 3 ? 12 : l == 4 ? 8 : l == 5 ? 6 : 5; }
+// Offset of level l's pixels among all levels' (the sums of the squared sides).
+__host__ __device__ constexpr int fused_off(int l) {
+    return l == 1 ? 0 : l == 2 ? 1156 : l == 3 ? 1556 : l == 4 ? 1700 : l == 5 ? 1764 : l == 6 ? 1800 : 1825;
+}
+
+// Keep threshold of coarse pixel (x, y) of a level held in shared memory (side s).
+__device__ __forceinline__ float keep_threshold(const float* M, const float* U, int s, int x, int y, float S) {
+    const float* m = M + y * s + x;
+    const float* u = U + y * s + x;
+    const float d = m[0];
+    bool edge = false;
+    if (d != INFINITY) {
+        const float nb[4] = {m[-1], m[1], m[-s], m[s]};
+        float te[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) te[e] = nb[e] == INFINITY ? 0.0f : __fsub_rn(nb[e], d);
+        const float lap = __fadd_rn(__fadd_rn(te[0], te[1]), __fadd_rn(te[2], te[3]));
+        edge = fabsf(lap) > __fmul_rn(kEdgeRel, d);
+    }
+    float ref = u[0];
+    if (edge) {
+        ref = INFINITY;
+#pragma unroll
+        for (int b = -1; b <= 1; ++b)
+#pragma unroll
+            for (int c = -1; c <= 1; ++c) ref = fminf(ref, u[b * s + c]);
+    }
+    return __fmul_rn(ref, S);
+}
+
+__global__ void __launch_bounds__(512) k_filter_fused(const FusedArgs a) {
+    constexpr int kTotal = fused_off(kMaxLevels + 1);
+    __shared__ float M[kTotal], U[kTotal];
+    __shared__ float thr[32 * 33];
+    const int bx = blockIdx.x, by = blockIdx.y;
+    // first pixel held of level l, per axis: tile * (32 >> (l - 1)) - (1 or 2)
+    auto origin = [](int b, int l) { return (b * 32 >> (l - 1)) - (l == 1 ? 1 : 2); };
+    // the tile's depth and every level's part in one round of loads
+    const int x = threadIdx.x & 63, gx = bx * 64 + x, gy0 = by * 64 + (threadIdx.x >> 6);
+    float depth[8], part[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        depth[i] = gx < a.W && gy0 + 8 * i < a.H ? a.depth[(size_t)(gy0 + 8 * i) * a.W + gx] : INFINITY;
+    static_assert(kTotal <= 4 * 512, "four positions a thread");
+    const int last = fused_off(a.n), total = fused_off(a.n + 1);  // level n's positions: [last, total)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = threadIdx.x + 512 * k;
+        if (i >= total) continue;
+        const int l = i < 1156 ? 1 : i < 1556 ? 2 : i < 1700 ? 3 : i < 1764 ? 4 : i < 1800 ? 5 : 6;
+        const int s = fused_side(l), r = i - fused_off(l), py = r / s, px = r - py * s;
+        const int qx = min(max(origin(bx, l) + px, 0), a.lev[l].W - 1), qy = min(max(origin(by, l) + py, 0), a.lev[l].H - 1);
+        part[k] = a.lev[l].M[(size_t)qy * a.lev[l].W + qx];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = threadIdx.x + 512 * k;
+        if (i >= total) continue;
+        M[i] = part[k];
+        if (i >= last) U[i] = part[k];
+    }
+    __syncthreads();
+    for (int l = a.n - 1; l >= 1; --l) {
+        const int s = fused_side(l), off = fused_off(l), sc = fused_side(l + 1), oc = fused_off(l + 1);
+        const int W = a.lev[l].W, H = a.lev[l].H;
+        for (int i = threadIdx.x; i < s * s; i += 512) {
+            const int x = min(max(origin(bx, l) + i % s, 0), W - 1), y = min(max(origin(by, l) + i / s, 0), H - 1);
+            const int cx = (x >> 1) - origin(bx, l + 1), cy = (y >> 1) - origin(by, l + 1);
+            const float m = M[off + i], t = keep_threshold(M + oc, U + oc, sc, cx, cy, a.S);
+            float val = INFINITY;
+            if (m <= t && m != INFINITY) {
+                val = m;
+            } else {  // fill: bilinear over the taps that are not empty
+                const float* u = U + oc + cy * sc + cx;
+                const int dx = x & 1 ? 1 : -1, dy = y & 1 ? sc : -sc;
+                const float tap[4] = {u[0], u[dx], u[dy], u[dy + dx]};
+                const float wt[4] = {0.5625f, 0.1875f, 0.1875f, 0.0625f};
+                float num = 0.0f, den = 0.0f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (tap[e] == INFINITY) continue;
+                    num = __fadd_rn(num, __fmul_rn(wt[e], tap[e]));
+                    den = __fadd_rn(den, wt[e]);
+                }
+                if (den > 0.0f) val = __fdiv_rn(num, den);
+            }
+            U[off + i] = val;
+        }
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < 1024; i += 512)
+        thr[(i >> 5) * 33 + (i & 31)] = keep_threshold(M, U, 34, (i & 31) + 1, (i >> 5) + 1, a.S);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int y = (threadIdx.x >> 6) + 8 * i;
+        if (gx < a.W && by * 64 + y < a.H)
+            a.kept[(size_t)(by * 64 + y) * a.W + gx] =
+                depth[i] <= thr[(y >> 1) * 33 + (x >> 1)] && depth[i] != INFINITY ? depth[i] : INFINITY;
     }
 }
 
@@ -922,38 +1062,26 @@ extern "C" lnr_status lnr_filter_static(const float* d_depth, int W, int H, int 
         scratch = g_static_ptr[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    ViewDev* view = reinterpret_cast<ViewDev*>(scratch);
-    float* M = scratch + kStaticViewFloats;
-    float* U = M + lev;
-    const float S = 1.0f + fs * 0.05f;  // keep scale, as for lnr_render
-    k_static_view<<<1, 1, 0, st>>>(view, S, 1.0f);
-    UpArgs a{};
-    a.views = view;
-    if (n_levels == 0) {
-        a.Mf = d_depth;
-        a.f_stride = (size_t)W * H;
-        a.Wf = W;
-        a.Hf = H;
-        a.u0 = d_kept;
-        k_pack_direct<2><<<2048, 256, 0, st>>>(a, 1);
+    if (n_levels == 0) {  // every filled pixel is kept
+        if (d_kept != d_depth &&
+            cudaMemcpyAsync(d_kept, d_depth, sizeof(float) * W * H, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+            return LNR_E_CUDA;
         return cudaGetLastError() == cudaSuccess ? LNR_OK : LNR_E_CUDA;
     }
-    dim3 g((W + 63) / 64, (H + 63) / 64, 1);
-    k_pyramid_from_depth<<<g, 256, 0, st>>>(d_depth, W, H, n_levels, M);
-    for (int l = n_levels - 1; l >= 0; --l) {
-        int Wl = W, Hl = H;
-        for (int k = 0; k < l; ++k) { Wl = (Wl + 1) / 2; Hl = (Hl + 1) / 2; }
-        UpArgs u = a;
-        u.Wf = Wl; u.Hf = Hl;
-        u.Wc = (Wl + 1) / 2; u.Hc = (Hl + 1) / 2;
-        u.Mf = l == 0 ? d_depth : M + pyramid_offset(W, H, l);
-        u.Mc = M + pyramid_offset(W, H, l + 1);
-        u.Uc = (l + 1 == n_levels) ? u.Mc : U + pyramid_offset(W, H, l + 1);
-        u.f_stride = u.c_stride = u.uc_stride = u.uf_stride = 0;
-        if (l > 0) { u.Uf = U + pyramid_offset(W, H, l); u.fill = 1; }
-        else { u.Uf = nullptr; u.u0 = d_kept; u.fill = 0; }
-        dim3 gu((u.Wc + 31) / 32, (u.Hc + 7) / 8, 1);
-        k_upsample<2><<<gu, 256, 0, st>>>(u);
+    FusedArgs a{};
+    a.depth = d_depth;
+    a.kept = d_kept;
+    a.W = W;
+    a.H = H;
+    a.n = n_levels;
+    a.S = 1.0f + fs * 0.05f;  // keep scale, as for lnr_render
+    for (int l = 1, w = W, h = H; l <= n_levels; ++l) {
+        w = (w + 1) / 2;
+        h = (h + 1) / 2;
+        a.lev[l] = FusedLevel{w, h, scratch + pyramid_offset(W, H, l)};
     }
+    const dim3 g((W + 63) / 64, (H + 63) / 64, 1);
+    k_pyramid_from_depth<<<g, 512, 0, st>>>(d_depth, W, H, n_levels, scratch);
+    k_filter_fused<<<g, 512, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? LNR_OK : LNR_E_CUDA;
 }
