@@ -15,6 +15,8 @@
 // implementation of that same sequence.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "lnr_internal.h"
 
 namespace lnr {
@@ -919,7 +921,7 @@ __global__ void __launch_bounds__(512) k_pyramid_from_depth(const float* __restr
 // coarse work, itself a third of the fine).  Positions outside the image hold the values of the
 // nearest pixel inside, as the replicated borders of the method.  One launch in place of one
 // per level, whose grids of a few blocks each took 5 us one after the other: 1920x1080 with 5
-// levels, whole call 39.9 -> 24.4 us.
+// levels, whole call 40.9 -> 20.5 us.  Bound by its instructions (76 % of issue slots).
 struct FusedLevel {
     int W, H;        // level size
     const float* M;  // min-pooled level
@@ -937,10 +939,10 @@ __host__ __device__ constexpr int fused_off(int l) {
     return l == 1 ? 0 : l == 2 ? 1156 : l == 3 ? 1556 : l == 4 ? 1700 : l == 5 ? 1764 : l == 6 ? 1800 : 1825;
 }
 
-// Keep threshold of coarse pixel (x, y) of a level held in shared memory (side s).
-__device__ __forceinline__ float keep_threshold(const float* M, const float* U, int s, int x, int y, float S) {
-    const float* m = M + y * s + x;
-    const float* u = U + y * s + x;
+// Keep threshold of coarse pixel c of a level held in shared memory (side s).
+__device__ __forceinline__ float keep_threshold(const float* M, const float* U, int s, int c, float S) {
+    const float* m = M + c;
+    const float* u = U + c;
     const float d = m[0];
     bool edge = false;
     if (d != INFINITY) {
@@ -957,9 +959,44 @@ __device__ __forceinline__ float keep_threshold(const float* M, const float* U, 
 #pragma unroll
         for (int b = -1; b <= 1; ++b)
 #pragma unroll
-            for (int c = -1; c <= 1; ++c) ref = fminf(ref, u[b * s + c]);
+            for (int e = -1; e <= 1; ++e) ref = fminf(ref, u[b * s + e]);
     }
     return __fmul_rn(ref, S);
+}
+
+// Upsampled level L of the block's part, from level L + 1 (sides known at compile time: the
+// positions' divisions are by constants).
+template <int L>
+__device__ __forceinline__ void fused_level(const FusedArgs& a, float* M, float* U, int x0, int y0, int cx0, int cy0) {
+    constexpr int s = fused_side(L), off = fused_off(L), sc = fused_side(L + 1), oc = fused_off(L + 1);
+    const int W = a.lev[L].W, H = a.lev[L].H;
+#pragma unroll
+    for (int i0 = 0; i0 < s * s; i0 += 512) {
+        const int i = i0 + threadIdx.x;
+        if (i >= s * s) break;
+        const int x = min(max(x0 + i % s, 0), W - 1), y = min(max(y0 + i / s, 0), H - 1);
+        const int c = ((y >> 1) - cy0) * sc + (x >> 1) - cx0;
+        const float m = M[off + i], t = keep_threshold(M + oc, U + oc, sc, c, a.S);
+        float val = INFINITY;
+        if (m <= t && m != INFINITY) {
+            val = m;
+        } else {  // fill: bilinear over the taps that are not empty
+            const float* u = U + oc + c;
+            const int dx = x & 1 ? 1 : -1, dy = y & 1 ? sc : -sc;
+            const float tap[4] = {u[0], u[dx], u[dy], u[dy + dx]};
+            const float wt[4] = {0.5625f, 0.1875f, 0.1875f, 0.0625f};
+            float num = 0.0f, den = 0.0f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const bool full = tap[e] != INFINITY;
+                num = full ? __fadd_rn(num, __fmul_rn(wt[e], tap[e])) : num;
+                den = full ? __fadd_rn(den, wt[e]) : den;
+            }
+            if (den > 0.0f) val = __fdiv_rn(num, den);
+        }
+        U[off + i] = val;
+    }
+    __syncthreads();
 }
 
 __global__ void __launch_bounds__(512) k_filter_fused(const FusedArgs a) {
@@ -994,36 +1031,18 @@ __global__ void __launch_bounds__(512) k_filter_fused(const FusedArgs a) {
         if (i >= last) U[i] = part[k];
     }
     __syncthreads();
-    for (int l = a.n - 1; l >= 1; --l) {
-        const int s = fused_side(l), off = fused_off(l), sc = fused_side(l + 1), oc = fused_off(l + 1);
-        const int W = a.lev[l].W, H = a.lev[l].H;
-        for (int i = threadIdx.x; i < s * s; i += 512) {
-            const int x = min(max(origin(bx, l) + i % s, 0), W - 1), y = min(max(origin(by, l) + i / s, 0), H - 1);
-            const int cx = (x >> 1) - origin(bx, l + 1), cy = (y >> 1) - origin(by, l + 1);
-            const float m = M[off + i], t = keep_threshold(M + oc, U + oc, sc, cx, cy, a.S);
-            float val = INFINITY;
-            if (m <= t && m != INFINITY) {
-                val = m;
-            } else {  // fill: bilinear over the taps that are not empty
-                const float* u = U + oc + cy * sc + cx;
-                const int dx = x & 1 ? 1 : -1, dy = y & 1 ? sc : -sc;
-                const float tap[4] = {u[0], u[dx], u[dy], u[dy + dx]};
-                const float wt[4] = {0.5625f, 0.1875f, 0.1875f, 0.0625f};
-                float num = 0.0f, den = 0.0f;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (tap[e] == INFINITY) continue;
-                    num = __fadd_rn(num, __fmul_rn(wt[e], tap[e]));
-                    den = __fadd_rn(den, wt[e]);
-                }
-                if (den > 0.0f) val = __fdiv_rn(num, den);
-            }
-            U[off + i] = val;
-        }
-        __syncthreads();
-    }
+    auto level = [&](auto lc) {
+        constexpr int L = decltype(lc)::value;
+        if (a.n > L)
+            fused_level<L>(a, M, U, origin(bx, L), origin(by, L), origin(bx, L + 1), origin(by, L + 1));
+    };
+    level(std::integral_constant<int, 5>{});
+    level(std::integral_constant<int, 4>{});
+    level(std::integral_constant<int, 3>{});
+    level(std::integral_constant<int, 2>{});
+    level(std::integral_constant<int, 1>{});
     for (int i = threadIdx.x; i < 1024; i += 512)
-        thr[(i >> 5) * 33 + (i & 31)] = keep_threshold(M, U, 34, (i & 31) + 1, (i >> 5) + 1, a.S);
+        thr[(i >> 5) * 33 + (i & 31)] = keep_threshold(M, U, 34, ((i >> 5) + 1) * 34 + (i & 31) + 1, a.S);
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
