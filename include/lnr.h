@@ -122,7 +122,7 @@ lnr_status lnr_set_precision(lnr_ctx* ctx, lnr_precision precision);
  *    the filter keeps (foreground) and the projected point colour / 255 for pixels it
  *    drops (background), D = z / zfar, A = 1; zero where no point falls.
  * out: host, H*W*5 FP32 (r, g, b, D, A).  The ground truth of the pair is gt itself.
- * Errors as lnr_render_stage; LNR_E_ARG for null gt_rgb / out.  Allocates temporaries. */
+ * Errors as lnr_render_stage; LNR_E_ARG for null gt_rgb / out. */
 lnr_status lnr_training_input(lnr_ctx* ctx, const lnr_view* view, const lnr_intrinsics* intr,
                               int W, int H, int n_levels, float fs, const float* gt_rgb,
                               int unfiltered, float* out);
