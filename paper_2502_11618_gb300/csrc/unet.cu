@@ -50,13 +50,26 @@ size_t unet_in_bytes_per_px(lnr_precision) { return 32; }
 // Bytes of an activation: three BF16 parts (conv_split.cu) for the FP32 network.
 static size_t elem_bytes(lnr_precision p) { return p == LNR_FP32 ? 6 : 2; }
 
+// Elements of a level's activation buffer k.  The FP32 network writes its decoder outputs over
+// the level's skip tensor, which no later conv reads, so that its 6 bytes per value take about
+// the memory that 4 took with a buffer of their own (the FP8 calibration reads the other
+// precisions' outputs after the frame).
+static size_t slot_elems(const Unet& u, int B, int W, int H, lnr_precision p, int l, int k) {
+    if (k == 3 && p == LNR_FP32) return 0;
+    if (k == 2) return (size_t)B * (W >> (l + 1)) * (H >> (l + 1)) * u.ch[l];
+    return (size_t)B * (W >> l) * (H >> l) * u.ch[l];
+}
+
 // Activation buffers of the forward pass (the network input and output are counted with the
 // frame's raster buffers): four per level, each at most the level's size (+ 256 bytes).
 size_t unet_act_bytes(const Unet& u, int B, int W, int H, lnr_precision p) {
     size_t tot = 0;
     for (int l = 0; l < u.levels; ++l) {
-        size_t Pl = (size_t)B * (W >> l) * (H >> l);
-        tot += (Pl * u.ch[l] * elem_bytes(p) + 256) * 4;
+        if (p != LNR_FP32) {
+            tot += (slot_elems(u, B, W, H, p, l, 0) * elem_bytes(p) + 256) * 4;
+            continue;
+        }
+        for (int k = 0; k < 4; ++k) tot += slot_elems(u, B, W, H, p, l, k) * elem_bytes(p) + 256;
     }
     return tot;
 }
@@ -67,9 +80,9 @@ cudaError_t unet_ensure(const Unet& u, Workspace& ws, lnr_precision p) {
     const size_t e = elem_bytes(p);
     cudaError_t err;
     for (int l = 0; l < u.levels; ++l) {
-        size_t Pl = (size_t)ws.B * (ws.W >> l) * (ws.H >> l);
         for (int k = 0; k < 4; ++k) {
-            size_t n = (k == 2) ? (size_t)ws.B * (ws.W >> (l + 1)) * (ws.H >> (l + 1)) * u.ch[l] : Pl * u.ch[l];
+            const size_t n = slot_elems(u, ws.B, ws.W, ws.H, p, l, k);
+            if (!n && k == 3) continue;
             const void* before = ws.act[slot(l, k)].p;
             if ((err = ws.act[slot(l, k)].ensure(n * e + 256))) return err;
             if (before != ws.act[slot(l, k)].p) ws.alloc_gen++;
@@ -114,7 +127,7 @@ static std::vector<ConvCall> unet_plan(const Unet& u, Workspace& ws, lnr_precisi
     for (int l = L - 2; l >= 0; --l) {
         const int W = ws.W >> l, H = ws.H >> l;
         void* t = ws.act[slot(l, 0)].p;
-        void* d = ws.act[slot(l, 3)].p;
+        void* d = ws.act[slot(l, p == LNR_FP32 ? 1 : 3)].p;
         const void* skip = ws.act[slot(l, 1)].p;
         calls.push_back({ci, skip, deep, t, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, W, H});
         const bool fuse_head = (l == 0) && p != LNR_FP32;
@@ -184,7 +197,7 @@ void unet_forward(const lnr_ctx* c, Workspace& ws, lnr_precision p, const void* 
         if (layer_ev) cudaEventRecord(layer_ev[ev++], st);
     }
     if (p == LNR_FP32) {
-        const void* deep = ws.act[slot(u.levels > 1 ? 0 : 0, u.levels > 1 ? 3 : 1)].p;
+        const void* deep = calls.back().out;
         size_t npx = (size_t)ws.B * ws.W * ws.H;
         const unsigned grid = (unsigned)std::min<size_t>((npx + 255) / 256, (size_t)c->num_sms * 8);
         k_head_f32<<<grid, 256, 0, st>>>((const float*)deep, split_head_parts(u.convs.back()), u.head_b, u.out_ch, out,
