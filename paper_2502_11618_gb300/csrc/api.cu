@@ -417,10 +417,14 @@ lnr_status lnr_load_cloud(lnr_ctx* c, const double* xyz, const uint8_t* rgb, con
     if ((e = c->xyz.ensure(24 * n)) || (e = c->rgbs_in.ensure(4 * n)) || (e = bytes.ensure((scan_id ? 4 : 3) * n)))
         return cuda_fail(c, e, "cloud upload");
     uint8_t* scan = scan_id ? bytes.as<uint8_t>() + 3 * n : nullptr;
-    if ((e = cudaMemcpy(c->xyz.p, xyz, 24 * n, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(bytes.p, rgb, 3 * n, cudaMemcpyHostToDevice)) ||
-        (scan_id && (e = cudaMemcpy(scan, scan_id, n, cudaMemcpyHostToDevice))) ||
+    // The copies go on the context's stream, ahead of the kernels that read them: cudaMemcpy from
+    // pageable memory may return with its DMA in flight, and this stream does not wait for the
+    // legacy stream.  pack_rgbs waits for all of it, so that the caller's arrays are free again.
+    if ((e = cudaMemcpyAsync(c->xyz.p, xyz, 24 * n, cudaMemcpyHostToDevice, c->stream)) ||
+        (e = cudaMemcpyAsync(bytes.p, rgb, 3 * n, cudaMemcpyHostToDevice, c->stream)) ||
+        (scan_id && (e = cudaMemcpyAsync(scan, scan_id, n, cudaMemcpyHostToDevice, c->stream))) ||
         (e = pack_rgbs(bytes.as<uint8_t>(), scan, n, c->rgbs_in.as<uint32_t>(), c->stream))) {
+        cudaStreamSynchronize(c->stream);
         bytes.release();
         return cuda_fail(c, e, "cloud upload");
     }
@@ -742,13 +746,21 @@ lnr_status lnr_render_stage(lnr_ctx* c, const lnr_view* view, const lnr_intrinsi
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     cudaError_t e = cudaSuccess;
     std::vector<uint8_t> tmp;
+    uint64_t totals[2];
+    // what was put together on the host goes out on the stream, which is waited for below
+    auto deliver = [&](const void* src, size_t n) {
+        if (on_device) return cudaMemcpyAsync(out, src, n, cudaMemcpyHostToDevice, ws.stream);
+        std::memcpy(out, src, n);
+        return cudaSuccess;
+    };
     switch (stage) {
         case LNR_STAGE_CULL: {
-            uint32_t t[2];
+            uint32_t t[2] = {0, 0};
             e = cudaMemcpyAsync(t, ws.vis_tot.p, 8, cudaMemcpyDeviceToHost, ws.stream);
             if (!e) e = cudaStreamSynchronize(ws.stream);
-            uint64_t r[2] = {t[0], t[1]};
-            if (!e) e = cudaMemcpy(out, r, 16, on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost);
+            totals[0] = t[0];
+            totals[1] = t[1];
+            if (!e) e = deliver(totals, 16);
             break;
         }
         case LNR_STAGE_KEYS:
@@ -765,7 +777,7 @@ lnr_status lnr_render_stage(lnr_ctx* c, const lnr_view* view, const lnr_intrinsi
                 std::memcpy(&tmp[8 * q], &d[q], 4);
                 std::memcpy(&tmp[8 * q + 4], &col[q], 4);
             }
-            if (!e) e = cudaMemcpy(out, tmp.data(), 8 * P, on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost);
+            if (!e) e = deliver(tmp.data(), 8 * P);
             break;
         }
         case LNR_STAGE_FILTERED:

@@ -1324,6 +1324,7 @@ static void tc_init() {
         cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
         cudaMalloc(&g_err, sizeof(int));
         cudaMemset(g_err, 0, sizeof(int));
+        cudaStreamSynchronize(nullptr);
         cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     }
 }

@@ -321,6 +321,9 @@ lnr_status unet_calibrate_fp8(lnr_ctx* c, Workspace& ws) {
         if ((e = tc_prepare_fp8(L)) != cudaSuccess) return cuda_fail(c, e, "FP8 weights");
         L.fp8 = true;
     }
+    // the weights' copies, from pageable memory on the legacy stream, are done before any frame
+    // on the context's stream reads them
+    if ((e = cudaStreamSynchronize(nullptr)) != cudaSuccess) return cuda_fail(c, e, "FP8 weights");
     u.fp8_ready = true;
     c->unet_gen++;
     return LNR_OK;

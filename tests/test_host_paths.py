@@ -1,0 +1,34 @@
+"""Host code of the library on a pretended CUDA runtime: order of copies and kernels, failed
+calls, several devices (no GPU; host_harness.py)."""
+from host_harness import run  # noqa: F401
+
+
+def test_uploads_are_ordered_before_the_kernels_that_read_them(run):  # noqa: F811
+    """A copy from pageable memory may still be in flight when cudaMemcpy returns, and the
+    context's stream does not wait for the legacy stream: clouds of few and many points, loaded
+    again on one context, with and without scanner ids, then each kind of call."""
+    run(r"""
+r = renderer()
+for n in (1, 100, 50_000):
+    xyz, rgb, sid = cloud(n, seed=n)
+    for s in (sid, None):
+        r.load_cloud(xyz, rgb, s)
+        assert get("unordered") == 0, ("load_cloud", n)
+        r.build_grid(0.5)
+        assert get("unordered") == 0, ("build_grid", n)
+r.render(VIEW, INTR, W, H, 2, 1.0)
+assert get("unordered") == 0, "fp32 frame"
+for stage in range(5):
+    r.render_stage(VIEW, INTR, W, H, 2, 1.0, stage)
+    out = Dev(20 * W * H)
+    assert fk.lnr_render_stage(r._c, ctypes.byref(_lib.make_view(VIEW)), ctypes.byref(_lib.make_intr(INTR)), W, H, 2,
+                               ctypes.c_float(1.0), stage, ctypes.c_void_p(out.data_ptr()), 1) == 0
+    assert get("unordered") == 0, ("stage", stage)
+r.set_precision("bf16")
+r.render(VIEW, INTR, W, H, 2, 1.0)
+r.calibrate(VIEW, INTR, W, H, 2, 1.0)
+r.set_precision("fp8")
+r.render(VIEW, INTR, W, H, 2, 1.0)
+assert get("unordered") == 0, "fp8 frame"
+assert get("launches") > 40
+""")
