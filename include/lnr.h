@@ -175,7 +175,8 @@ lnr_status lnr_set_soft_zbuffer(lnr_ctx* ctx, float rel);
 /* Render one frame (Fig. 1): cull, splat, filter (Fig. 2) with n_levels min-pool levels
  * and filter_strength fs, U-Net.  out_rgb: H*W*3 FP32 in [0, 1], HWC; host memory, or
  * device memory when out_on_device != 0 (then the call returns without waiting for the
- * GPU; the result is complete when the context's stream reaches it).
+ * GPU; the result is complete when the context's stream reaches it, and a bounded wait that
+ * ran out on the device fails this context's next render that does wait, LNR_E_TIMEOUT).
  * Errors: LNR_E_STATE before build_grid / set_unet; LNR_E_ARG when W or H is not a
  * positive multiple of 2^(levels-1), n_levels is outside [0, floor(log2(min(W, H)))] or
  * above 6, fs is negative or NaN, or the view is not finite. */

@@ -26,6 +26,13 @@ lnr_status cuda_fail(lnr_ctx* c, cudaError_t e, const char* where) {
                 std::string(where) + ": " + cudaGetErrorString(e));
 }
 
+lnr_status tc_error_status(int code) { return code >= 5 && code <= 7 ? LNR_E_TIMEOUT : LNR_E_CUDA; }
+
+std::string tc_error_text(int code) {
+    if (tc_error_status(code) == LNR_E_TIMEOUT) return "a tensor-core kernel gave up waiting (bounded wait ran out)";
+    return "a tensor-core convolution could not be launched (code " + std::to_string(code) + ")";
+}
+
 void Workspace::release() {
     DBuf* all[] = {&view, &cull_flag, &cull_cnt, &cull_bsum, &vis_info, &vis_pref, &vis_tot, &chunk_cell, &keys,
                    &soft_acc, &depth, &rgba, &pyr_m, &pyr_u, &u0, &out};
@@ -43,6 +50,7 @@ void Workspace::release() {
     for (auto& kv : graphs) cudaGraphExecDestroy(kv.second);
     graphs.clear();
     graph_uses.clear();
+    tc.release();
 }
 
 size_t Workspace::device_bytes() const {
@@ -118,6 +126,7 @@ static cudaError_t ensure_ws(const lnr_ctx* c, Workspace& ws, int B, int W, int 
                             ws.vis_tot.p, ws.depth.p, ws.rgba.p, ws.pyr_m.p, ws.pyr_u.p, ws.u0.p, ws.out.p, ws.keys.p,
                             ws.soft_acc.p, ws.chunk_cell.p};
     const size_t P = (size_t)W * H;
+    if ((e = ws.tc.ensure(c->num_sms))) return e;
     const int nb = cull_blocks(c->ncells);
     const size_t pf = pyramid_floats(W, H, kMaxLevels);
     if ((e = ws.view.ensure(sizeof(ViewDev) * B)) || (e = ws.cull_flag.ensure(4 * c->ncells * B)) ||
@@ -338,9 +347,8 @@ static lnr_status finish_output(lnr_ctx* c, Workspace& ws, float* out, size_t nf
     }
     if (c->timing) read_timing(c, ws);
     if (!on_device || c->timing) {
-        const int w = tc_error_word();
-        if (w >= 5 && w <= 7) return fail(c, LNR_E_TIMEOUT, "a tensor-core kernel gave up waiting (bounded wait ran out)");
-        if (w) return fail(c, LNR_E_CUDA, "a tensor-core convolution could not be launched (code " + std::to_string(w) + ")");
+        const int w = ws.tc.take();
+        if (w) return fail(c, tc_error_status(w), tc_error_text(w));
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "render launch");
@@ -537,9 +545,8 @@ lnr_status lnr_shard_finish(lnr_ctx* c, const lnr_view* view, const lnr_intrinsi
     if (!e) e = cudaStreamSynchronize(ws.stream);
     if (!e) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "shard_finish");
-    const int w = tc_error_word();
-    if (w >= 5 && w <= 7) return fail(c, LNR_E_TIMEOUT, "a tensor-core kernel gave up waiting (bounded wait ran out)");
-    if (w) return fail(c, LNR_E_CUDA, "a tensor-core convolution could not be launched (code " + std::to_string(w) + ")");
+    const int w = ws.tc.take();
+    if (w) return fail(c, tc_error_status(w), tc_error_text(w));
     return LNR_OK;
 }
 
@@ -843,6 +850,7 @@ lnr_status lnr_autotune(lnr_ctx* c, int W, int H, int batch) {
     const void* out_before = ws.out.p;
     if (!e) e = ws.act[4 * kMaxUnetLevels].ensure((size_t)batch * W * H * unet_in_bytes_per_px(c->prec) + 256);
     if (!e) e = ws.out.ensure((size_t)batch * W * H * 12);
+    if (!e) e = ws.tc.ensure(c->num_sms);
     if (!e) e = unet_ensure(c->unet, ws, c->prec);
     if (e != cudaSuccess) return cuda_fail(c, e, "autotune buffers");
     if (in_before != ws.act[4 * kMaxUnetLevels].p || out_before != ws.out.p) ws.alloc_gen++;

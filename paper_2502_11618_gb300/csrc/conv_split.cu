@@ -502,7 +502,7 @@ void pick_tile(const ConvLayer& L, int NT, int B, int W, int H, int num_sms, int
         }
 }
 
-void launch(void (*kern)(SParams), const SParams& p, int grid, size_t smem, cudaStream_t st) {
+void launch(void (*kern)(SParams), const SParams& p, int grid, size_t smem, cudaStream_t st, TcState& tc) {
     static std::mutex mu;
     static std::set<const void*> done;
     {
@@ -512,7 +512,7 @@ void launch(void (*kern)(SParams), const SParams& p, int grid, size_t smem, cuda
     }
     kern<<<grid, kSplitThreads, smem, st>>>(p);
     count_launch();
-    if (cudaGetLastError() != cudaSuccess) tc_host_error(9);
+    if (cudaGetLastError() != cudaSuccess) tc.host_err = 9;
 }
 
 }  // namespace
@@ -566,10 +566,10 @@ cudaError_t split_prepare_layer(ConvLayer& L) {
 int split_head_parts(const ConvLayer& L) { return 2 * (L.cout / tile_channels(L)); }
 
 void conv_split(const ConvLayer& L, const void* src0, const void* src1, void* out, void* pool_out, float* logits,
-                const float* head_wh, int head_o, int B, int W, int H, cudaStream_t st) {
+                const float* head_wh, int head_o, int B, int W, int H, cudaStream_t st, TcState& tc) {
     SParams p;
     std::memset(&p, 0, sizeof(p));
-    const int N = L.cout, NT = tile_channels(L), num_sms = tc_num_sms();
+    const int N = L.cout, NT = tile_channels(L), num_sms = tc.num_sms;
     int R = 0, P = 0;
     pick_tile(L, NT, B, W, H, num_sms, R, P);
     p.packed = L.cin0 == 5;
@@ -632,17 +632,17 @@ void conv_split(const ConvLayer& L, const void* src0, const void* src1, void* ou
     p.head_o = head_o;
     if (logits)
         for (int i = 0; i < head_o * N; ++i) p.head[i] = head_wh[i];
-    p.err = tc_err_ptr();
+    p.err = tc.err;
     for (int i = 0; i < N; ++i) p.bias[i] = L.bf[i];
     if (!ok) {
-        tc_host_error(4);
+        tc.host_err = 4;
         return;
     }
     const size_t smem = 1024 + (size_t)p.a_slots * p.a_slot + (size_t)kBSlots * p.b_slot +
                         8 * (2 * p.a_slots + 2 * kBSlots + 6);
     const int grid = std::min(p.ntiles, num_sms);
     auto go = [&](auto r, auto par, auto nt) {
-        launch(k_conv_split<decltype(r)::value, decltype(par)::value, decltype(nt)::value>, p, grid, smem, st);
+        launch(k_conv_split<decltype(r)::value, decltype(par)::value, decltype(nt)::value>, p, grid, smem, st, tc);
     };
     using std::integral_constant;
     auto tile = [&](auto nt) {
@@ -668,7 +668,7 @@ void conv_split(const ConvLayer& L, const void* src0, const void* src1, void* ou
                 if (R == 1) return go(r1, r4, nt);
             if constexpr (8 * T <= 256) return go(r2, r4, nt);
         }
-        tc_host_error(8);
+        tc.host_err = 8;
     };
     switch (NT) {
         case 16: return tile(integral_constant<int, 16>{});

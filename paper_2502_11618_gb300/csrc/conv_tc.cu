@@ -1280,10 +1280,6 @@ bool encode(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t* dims, c
     return r == CUDA_SUCCESS;
 }
 
-int g_num_sms = 0;
-int* g_err = nullptr;
-int g_host_err = 0;  // host-side failure of a launch: 4 tensor map, 8 no FP8 configuration, 9 launch refused
-
 }  // namespace
 
 bool tc_available() { return true; }
@@ -1317,21 +1313,9 @@ cudaError_t tc_prepare_layer(ConvLayer& L, lnr_precision p) {
     return cudaSuccess;
 }
 
-static void tc_init() {
-    if (!g_num_sms) {
-        int dev;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaMalloc(&g_err, sizeof(int));
-        cudaMemset(g_err, 0, sizeof(int));
-        cudaStreamSynchronize(nullptr);
-        cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    }
-}
-
 static void tc_conv_generic(const ConvLayer& L, const void* src0, const void* src1, void* out, void* pool_out,
                             const float* head_w, const float* head_b, float* head_out, int B, int W, int H, int head_o,
-                            cudaStream_t st) {
+                            cudaStream_t st, TcState& tc) {
     Params p;
     std::memset(&p, 0, sizeof(p));
     const int N = L.cout;
@@ -1356,17 +1340,17 @@ static void tc_conv_generic(const ConvLayer& L, const void* src0, const void* sr
             cuuint64_t dims[5] = {(cuuint64_t)C, 2, (cuuint64_t)Ws / 2, (cuuint64_t)Hs, (cuuint64_t)B};
             cuuint64_t str[4] = {C * eb, 2 * C * eb, (cuuint64_t)Ws * C * eb, (cuuint64_t)Hs * Ws * C * eb};
             cuuint32_t box[5] = {(cuuint32_t)s.kc, 1, 128, 1, 1};
-            if (!encode(&s.a, 5, src, dims, str, box, s.kc)) g_host_err = 4;
+            if (!encode(&s.a, 5, src, dims, str, box, s.kc)) tc.host_err = 4;
         } else {
             cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)Ws, (cuuint64_t)Hs, (cuuint64_t)B};
             cuuint64_t str[3] = {C * eb, (cuuint64_t)Ws * C * eb, (cuuint64_t)Hs * Ws * C * eb};
             cuuint32_t box[4] = {(cuuint32_t)s.kc, kind == 0 ? 64u : 128u, kind == 0 ? 2u : 1u, 1};
-            if (!encode(&s.a, 4, src, dims, str, box, s.kc)) g_host_err = 4;
+            if (!encode(&s.a, 4, src, dims, str, box, s.kc)) tc.host_err = 4;
         }
         cuuint64_t wd[2] = {Ktot, (cuuint64_t)N};
         cuuint64_t ws_[1] = {Ktot * eb};
         cuuint32_t wb[2] = {(cuuint32_t)s.kc, (cuuint32_t)N};
-        if (!encode(&s.b, 2, L.wtc, wd, ws_, wb, s.kc)) g_host_err = 4;
+        if (!encode(&s.b, 2, L.wtc, wd, ws_, wb, s.kc)) tc.host_err = 4;
     };
     if (p.parity) {
         p.nseg = 2;
@@ -1401,10 +1385,12 @@ static void tc_conv_generic(const ConvLayer& L, const void* src0, const void* sr
     p.head_b = head_b;
     p.head_out = head_out;
     p.head_o = head_o;
-    p.err = g_err;
+    p.err = tc.err;
     const size_t smem = 1024 + (size_t)p.stages * p.stage_bytes + p.xch_bytes + 8 * (2 * p.stages + 6) + 16;
-    const int grid = std::min(p.ntiles, g_num_sms);
-    if (g_host_err || !L.wtc) return;
+    const int grid = std::min(p.ntiles, tc.num_sms);
+    if (tc.host_err || !L.wtc) return;
+    static std::once_flag once;
+    std::call_once(once, [] { cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); });
     k_conv_tc<<<grid, kThreads, smem, st>>>(p);
     count_launch();
 }
@@ -1670,7 +1656,7 @@ struct HaloTypes {
 // head_wh, head_bh: host copies of the fused head's weights [head_o][N] and biases.
 bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* out, void* pool_out,
                   const float* head_wh, const float* head_bh, float* head_out, int B, int W, int H, int head_o, int R,
-                  int P, int ckmax, int O, int E, cudaStream_t st, const HaloTypes& ty = HaloTypes()) {
+                  int P, int ckmax, int O, int E, cudaStream_t st, const HaloTypes& ty, TcState& tc) {
     const int esize = ty.in8 ? 1 : 2;
     if (L.cout > kHaloMaxN || (int)L.bf.size() < L.cout || (head_out && (head_o > 4 || !head_wh || !head_bh)))
         return false;
@@ -1806,7 +1792,7 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
     (void)halo_stage_bytes;
     if (p.stages < 2) return false;
     if (!ok) {
-        g_host_err = 4;
+        tc.host_err = 4;
         return true;
     }
     p.tbufs = 2 * NC * R * N <= 512 ? 2 : 1;
@@ -1832,7 +1818,7 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
     p.inv_out = ty.inv_out;
     p.head_out = head_out;
     p.head_o = head_o;
-    p.err = g_err;
+    p.err = tc.err;
     const size_t smem = 1024 + (size_t)p.stages * p.stage_bytes + stg_total + 8 * (2 * p.stages + 7) + 16;
     // LNR_TEST_STALL_ONCE=1: the first halo launch of the process waits on a barrier nothing
     // arrives on and gives up after ~1 ms; the others then give up after ~2 s (the test of
@@ -1842,7 +1828,7 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
         return e && atoi(e) == 1 ? 1 : 0;
     }()};
     if (stall_once.exchange(0)) p.stall = 1;
-    const int grid = std::min(p.ntiles, g_num_sms);
+    const int grid = std::min(p.ntiles, tc.num_sms);
     auto launch = [&](void (*kern)(HParams), int threads) {
         static std::mutex mu;
         static std::set<const void*> done;
@@ -1853,7 +1839,7 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
         }
         kern<<<grid, threads, smem, st>>>(p);
         count_launch();
-        if (cudaGetLastError() != cudaSuccess) g_host_err = 9;  // a launch that did not start: reported, never silent
+        if (cudaGetLastError() != cudaSuccess) tc.host_err = 9;  // a launch that did not start: reported, never silent
     };
     auto pick4 = [&](auto par, auto ep) {
         constexpr int PP = decltype(par)::value, EE = decltype(ep)::value;
@@ -1905,8 +1891,7 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
 // second conv L1 with its 2x2 pooled output.  R output rows per tile (2 or 4).  Returns false
 // when the pair or the types do not fit it (the caller then runs the two convs apart).
 bool tc_enc0_fused(const ConvLayer& L0, const ConvLayer& L1, const void* in, void* out, void* pool_out, int B, int W,
-                   int H, int R, cudaStream_t st, const HaloTypes& ty1) {
-    tc_init();
+                   int H, int R, cudaStream_t st, const HaloTypes& ty1, TcState& tc) {
     const int N1 = L0.cout, N2 = L1.cout;
     if (L0.cin0 != 5 || L0.cin1 || L1.cin0 != N1 || L1.cin1 || !L1.pool || !pool_out || (N1 != 16 && N1 != 32) ||
         (N2 != 16 && N2 != 32) || (R != 2 && R != 4) || ty1.in8 || ty1.out8)
@@ -1951,7 +1936,7 @@ bool tc_enc0_fused(const ConvLayer& L0, const ConvLayer& L1, const void* in, voi
     p.pool_out = pool_out;
     p.pool8 = ty1.pool8 ? 1 : 0;
     p.inv_pool = ty1.inv_out;
-    p.err = g_err;
+    p.err = tc.err;
     cuuint32_t es[5] = {1, 1, 1, 1, 1};
     bool ok;
     {
@@ -1963,11 +1948,11 @@ bool tc_enc0_fused(const ConvLayer& L0, const ConvLayer& L1, const void* in, voi
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
     if (!ok) {
-        g_host_err = 4;
+        tc.host_err = 4;
         return true;
     }
     const size_t smem = 1024 + (size_t)p.act_off + 2 * p.act_bytes + 8 * (2 * p.stages + 14) + 16;
-    const int grid = std::min(p.ntiles, g_num_sms);
+    const int grid = std::min(p.ntiles, tc.num_sms);
     auto launch = [&](void (*kern)(FParams)) {
         static std::mutex mu;
         static std::set<const void*> done;
@@ -1978,7 +1963,7 @@ bool tc_enc0_fused(const ConvLayer& L0, const ConvLayer& L1, const void* in, voi
         }
         kern<<<grid, kFuseThreads, smem, st>>>(p);
         count_launch();
-        if (cudaGetLastError() != cudaSuccess) g_host_err = 9;
+        if (cudaGetLastError() != cudaSuccess) tc.host_err = 9;
     };
     if (R == 2) launch(k_enc0_fused<2>);
     else launch(k_enc0_fused<4>);
@@ -1989,7 +1974,7 @@ bool tc_enc0_fused(const ConvLayer& L0, const ConvLayer& L1, const void* in, voi
 // for both (FP8 mode keeps them BF16 by its policy); the pooled output stores E4M3 when its
 // consumer reads E4M3.
 bool tc_fused_enc0(const ConvLayer& L0, const ConvLayer& L1, lnr_precision prec, const void* in, void* out,
-                   void* pool_out, int B, int W, int H, int R, cudaStream_t st) {
+                   void* pool_out, int B, int W, int H, int R, cudaStream_t st, TcState& tc) {
     HaloTypes ty;
     if (prec == LNR_FP8) {
         if (L0.fp8 || L1.fp8) return false;
@@ -1997,7 +1982,7 @@ bool tc_fused_enc0(const ConvLayer& L0, const ConvLayer& L1, lnr_precision prec,
         ty.pool8 = !L1.pool_bf16;
         ty.inv_out = 1.0f / L1.out_scale;
     }
-    return tc_enc0_fused(L0, L1, in, out, pool_out, B, W, H, R, st, ty);
+    return tc_enc0_fused(L0, L1, in, out, pool_out, B, W, H, R, st, ty, tc);
 }
 
 // Whether a test's environment switch asks for one kernel variant everywhere: the untuned
@@ -2010,8 +1995,7 @@ bool tc_variant_forced() {
 
 void tc_conv(const ConvLayer& L, lnr_precision prec, const void* src0, const void* src1, void* out, void* pool_out,
              const float* head_w, const float* head_b, const float* head_wh, const float* head_bh, float* head_out, int B,
-             int W, int H, int head_o, cudaStream_t st, const TcConfig* force) {
-    tc_init();
+             int W, int H, int head_o, cudaStream_t st, TcState& tc, const TcConfig* force) {
     static const int forced = [] {
         const char* e = getenv("LNR_CONV_KERNEL");
         return (e && !strcmp(e, "generic")) ? 2 : (e && !strcmp(e, "halo")) ? 3 : 0;
@@ -2050,9 +2034,9 @@ void tc_conv(const ConvLayer& L, lnr_precision prec, const void* src0, const voi
             halo_default(L, R, P, CK);
             if (ty.in8) CK = std::max(32, CK);
             int E = 8;
-            if (!tc_variant_forced() && halo_pick(L, ty.in8 ? 1 : 2, CK, B, W, H, g_num_sms, R, P, E) &&
+            if (!tc_variant_forced() && halo_pick(L, ty.in8 ? 1 : 2, CK, B, W, H, tc.num_sms, R, P, E) &&
                 tc_conv_halo(L, src0, src1, out, pool_out, head_wh, head_bh, head_out, B, W, H, head_o, R, P, CK, 0, E, st,
-                             ty))
+                             ty, tc))
                 return;
             // a forced variant (tests): TMA-store epilogue where it fits next to two pipeline stages
             // LNR_CONV_TMA_STORE=0: direct stores; =1: one staging buffer per warp
@@ -2063,18 +2047,18 @@ void tc_conv(const ConvLayer& L, lnr_precision prec, const void* src0, const voi
             if (tma_store > 0)
                 for (int nbuf = std::min(tma_store, 2); nbuf >= 1; --nbuf)
                     if (tc_conv_halo(L, src0, src1, out, pool_out, head_wh, head_bh, head_out, B, W, H, head_o, R, P, CK, nbuf,
-                                     epi, st, ty))
+                                     epi, st, ty, tc))
                         return;
         }
         if (tc_conv_halo(L, src0, src1, out, pool_out, head_wh, head_bh, head_out, B, W, H, head_o, R, P, CK, cfg.O,
-                         cfg.mode == 0 ? epi : cfg.E, st, ty))
+                         cfg.mode == 0 ? epi : cfg.E, st, ty, tc))
             return;
         if (fp8) {  // no fallback for FP8: record and skip
-            g_host_err = 8;
+            tc.host_err = 8;
             return;
         }
     }
-    tc_conv_generic(L, src0, src1, out, pool_out, head_w, head_b, head_out, B, W, H, head_o, st);
+    tc_conv_generic(L, src0, src1, out, pool_out, head_w, head_b, head_out, B, W, H, head_o, st, tc);
 }
 
 // Every valid kernel configuration of a layer: the generic kernel, and the halo kernel over
@@ -2129,29 +2113,26 @@ std::vector<TcConfig> tc_candidates(const ConvLayer& L, lnr_precision prec) {
     return out;
 }
 
-int* tc_err_ptr() {
-    tc_init();
-    return g_err;
+cudaError_t TcState::ensure(int sms) {
+    num_sms = sms;
+    if (err) return cudaSuccess;
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&err), sizeof(int), cudaHostAllocPortable);
+    if (e == cudaSuccess) *err = 0;
+    return e;
 }
 
-int tc_num_sms() {
-    tc_init();
-    return g_num_sms;
+void TcState::release() {
+    if (err) cudaFreeHost(err);
+    err = nullptr;
 }
 
-void tc_host_error(int code) { g_host_err = code; }
-
-int tc_error_word() {
-    if (g_host_err) {
-        const int h = g_host_err;
-        g_host_err = 0;
-        return h;
-    }
-    if (!g_err) return 0;
-    int h = 0;
-    cudaMemcpy(&h, g_err, sizeof(int), cudaMemcpyDeviceToHost);
-    if (h) cudaMemset(g_err, 0, sizeof(int));
-    return h;
+int TcState::take() {
+    int code = host_err;
+    host_err = 0;
+    if (!err) return code;
+    if (!code) code = *static_cast<volatile int*>(err);
+    *static_cast<volatile int*>(err) = 0;
+    return code;
 }
 
 }  // namespace lnr

@@ -134,6 +134,17 @@ struct GraphKey {
     }
 };
 
+// What the tensor-core launches of one workspace share.  Nothing of it is shared between
+// workspaces, so that an error is reported for the frame that met it.
+struct TcState {
+    int num_sms = 0;
+    int* err = nullptr;  // page-locked, which kernels write: the bounded wait that ran out (5, 6 or 7), 0 none
+    int host_err = 0;    // on the host: 4 tensor map, 8 no FP8 configuration, 9 launch refused
+    cudaError_t ensure(int sms);
+    void release();
+    int take();  // the error since the last call, 0 none; the workspace's stream has been waited for
+};
+
 // Per-launch workspace: everything one batch of views needs on the device.
 struct Workspace {
     int B = 0, W = 0, H = 0, nlev = 0;
@@ -151,6 +162,7 @@ struct Workspace {
     DBuf act[4 * kMaxUnetLevels + 2];       // U-Net activations; [4 * kMaxUnetLevels] = U-Net input
     DBuf out;                               // float [B][P][3]
     float* out_ptr = nullptr;               // U-Net output of the next frame: a caller's device buffer, or null for out
+    TcState tc;
     bool allow_fuse = true;                 // false: every conv runs apart (the FP8 calibration frame reads every output)
     // View parameters go up from two pinned host blocks in turn; view_ev[k] is recorded right
     // after block k's upload, so composing the next frame waits only for the upload that
@@ -229,6 +241,8 @@ namespace lnr {
 double now_s();
 lnr_status fail(lnr_ctx* c, lnr_status s, const std::string& msg);
 lnr_status cuda_fail(lnr_ctx* c, cudaError_t e, const char* where);
+lnr_status tc_error_status(int code);  // of a TcState error
+std::string tc_error_text(int code);
 
 // grid.cu
 cudaError_t grid_bbox(const double* xyz, uint64_t n, long long* box, double out_lohi[6], cudaStream_t st);
@@ -285,16 +299,13 @@ bool tc_available();
 cudaError_t tc_prepare_layer(ConvLayer& L, lnr_precision p);
 void tc_conv(const ConvLayer& L, lnr_precision p, const void* src0, const void* src1, void* out, void* pool_out,
              const float* head_w, const float* head_b, const float* head_wh, const float* head_bh, float* head_out, int B,
-             int W, int H, int head_o, cudaStream_t st, const TcConfig* force = nullptr);
+             int W, int H, int head_o, cudaStream_t st, TcState& tc, const TcConfig* force = nullptr);
 std::vector<TcConfig> tc_candidates(const ConvLayer& L, lnr_precision p);
 // The first two encoder convs fused (R rows per tile, 2 or 4); false when they cannot be.
 bool tc_fused_enc0(const ConvLayer& L0, const ConvLayer& L1, lnr_precision p, const void* in, void* out,
-                   void* pool_out, int B, int W, int H, int R, cudaStream_t st);
+                   void* pool_out, int B, int W, int H, int R, cudaStream_t st, TcState& tc);
 cudaError_t tc_prepare_fp8(ConvLayer& L);
 std::vector<uint16_t> halo_blocks(const ConvLayer& L, int sg);  // weight blocks of a K segment, as tap masks
-int* tc_err_ptr();             // device error word of the bounded waits
-int tc_num_sms();
-void tc_host_error(int code);  // a launch that failed on the host: the next tc_error_word reports it
 bool tc_variant_forced();  // an LNR_CONV_* switch of the tests asks for one kernel variant
 
 // conv_split.cu: the FP32 network's convolutions.  Sources and outputs are [image][hi, mid,
@@ -304,7 +315,6 @@ bool tc_variant_forced();  // an LNR_CONV_* switch of the tests asks for one ker
 cudaError_t split_prepare_layer(ConvLayer& L);
 int split_head_parts(const ConvLayer& L);
 void conv_split(const ConvLayer& L, const void* src0, const void* src1, void* out, void* pool_out, float* logits,
-                const float* head_wh, int head_o, int B, int W, int H, cudaStream_t st);
-int tc_error_word();  // nonzero after a bounded wait in a tensor-core kernel ran out (then reset)
+                const float* head_wh, int head_o, int B, int W, int H, cudaStream_t st, TcState& tc);
 
 }  // namespace lnr

@@ -132,7 +132,8 @@ struct ServeReq {
     int W, H, nlev;
     float fs;
     double t_submit = 0, t_done = 0;
-    bool done = false, failed = false;
+    bool done = false;
+    lnr_status status = LNR_OK;
     float* host = nullptr;  // pinned result, H*W*3 floats
     size_t bytes = 0;
     float* user = nullptr;  // lnr_submit_into: the caller's destination
@@ -259,16 +260,19 @@ void Server::loop() {
             const cudaError_t q = cudaEventQuery(s.done);
             if (q == cudaErrorNotReady) continue;
             const double t = now_s();
+            const int w = q == cudaSuccess ? s.ws.tc.take() : 0;  // the frame is done: what its kernels met
+            const lnr_status st = q != cudaSuccess ? LNR_E_CUDA : w ? tc_error_status(w) : LNR_OK;
             std::lock_guard<std::mutex> g(mu);
             for (uint64_t tk : s.tickets) {
                 auto it = reqs.find(tk);
                 if (it == reqs.end()) continue;
                 it->second.done = true;
-                it->second.failed = q != cudaSuccess;
+                it->second.status = st;
                 it->second.t_done = t;
                 ++n_done;
             }
             if (q != cudaSuccess) err = cudaGetErrorString(q);
+            else if (w) err = tc_error_text(w);
             s.busy = false;
             s.tickets.clear();
             progressed = true;
@@ -307,7 +311,7 @@ void Server::loop() {
                 std::lock_guard<std::mutex> g(mu);
                 for (uint64_t tk : batch) {
                     reqs[tk].done = true;
-                    reqs[tk].failed = true;
+                    reqs[tk].status = LNR_E_CUDA;
                 }
                 err = c->err.empty() ? "launch failed" : c->err;
                 s.busy = false;
@@ -474,7 +478,7 @@ lnr_status lnr_poll(lnr_ctx* c, uint64_t ticket, float* out, double* latency_s) 
     }
     lnr_status st = LNR_OK;
     if (!out && !r.user_pinned) out = r.user;  // lnr_submit_into with a pageable destination
-    if (r.failed) st = fail(c, LNR_E_CUDA, "request failed: " + s->err);
+    if (r.status != LNR_OK) st = fail(c, r.status, "request failed: " + s->err);
     else if (out && r.host) s->copier.copy(out, r.host, r.bytes);
     else if (out && r.user_pinned && out != r.user) std::memcpy(out, r.user, r.bytes);
     if (latency_s) *latency_s = r.t_done - r.t_submit;

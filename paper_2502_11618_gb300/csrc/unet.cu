@@ -146,10 +146,10 @@ static void run_call(const Unet& u, const ConvCall& k, Workspace& ws, lnr_precis
     if (p == LNR_FP32)
         conv_split(L, k.src0, k.src1, k.out, k.pool,
                    k.layer + 1 == (int)u.convs.size() ? static_cast<float*>(k.out) : nullptr, u.head_wh.data(), u.out_ch,
-                   ws.B, k.W, k.H, st);
+                   ws.B, k.W, k.H, st, ws.tc);
     else
         tc_conv(L, p, k.src0, k.src1, k.out, k.pool, k.head_w, k.head_b, k.head_wh, k.head_bh, k.head_out, ws.B, k.W, k.H,
-                u.out_ch, st, force);
+                u.out_ch, st, ws.tc, force);
 }
 
 // Rows per tile of the fused level-0 encoder for B images at the layer resolution (W, H), or
@@ -186,7 +186,7 @@ void unet_forward(const lnr_ctx* c, Workspace& ws, lnr_precision p, const void* 
         if (k.layer == 0 && i + 1 < calls.size() && ws.allow_fuse) {
             const int R = fuse_rows(u, p, ws.B, k.W, k.H);
             const ConvCall& k1 = calls[i + 1];
-            if (R && tc_fused_enc0(u.convs[0], u.convs[1], p, k.src0, k1.out, k1.pool, ws.B, k.W, k.H, R, st)) {
+            if (R && tc_fused_enc0(u.convs[0], u.convs[1], p, k.src0, k1.out, k1.pool, ws.B, k.W, k.H, R, st, ws.tc)) {
                 ++i;  // both convs done
                 if (layer_ev) cudaEventRecord(layer_ev[ev++], st);
                 if (layer_ev) cudaEventRecord(layer_ev[ev++], st);
@@ -363,7 +363,7 @@ lnr_status unet_autotune(lnr_ctx* c, Workspace& ws, lnr_precision p, int reps) {
             if ((e = cudaEventSynchronize(e1)) != cudaSuccess) break;
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (tc_error_word()) continue;  // a configuration that failed is never chosen
+            if (ws.tc.take()) continue;  // a configuration that failed is never chosen
             if (log >= 2)
                 fprintf(stderr, "  candidate layer %d: mode %d R %d P %d ck %d O %d E %d  %.1f us\n", k.layer, cfg.mode,
                         cfg.R, cfg.P, cfg.CK, cfg.O, cfg.E, 1e3 * ms / reps);
@@ -386,15 +386,15 @@ lnr_status unet_autotune(lnr_ctx* c, Workspace& ws, lnr_precision p, int reps) {
         entry.F = 0;
         float best = best_ms[0] + best_ms[1];
         for (int R : {2, 4}) {
-            if (!tc_fused_enc0(u.convs[0], u.convs[1], p, k0.src0, k1.out, k1.pool, ws.B, k0.W, k0.H, R, st)) continue;
+            if (!tc_fused_enc0(u.convs[0], u.convs[1], p, k0.src0, k1.out, k1.pool, ws.B, k0.W, k0.H, R, st, ws.tc)) continue;
             cudaEventRecord(e0, st);
             for (int r = 0; r < reps; ++r)
-                tc_fused_enc0(u.convs[0], u.convs[1], p, k0.src0, k1.out, k1.pool, ws.B, k0.W, k0.H, R, st);
+                tc_fused_enc0(u.convs[0], u.convs[1], p, k0.src0, k1.out, k1.pool, ws.B, k0.W, k0.H, R, st, ws.tc);
             cudaEventRecord(e1, st);
             if ((e = cudaEventSynchronize(e1)) != cudaSuccess) break;
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (tc_error_word()) continue;
+            if (ws.tc.take()) continue;
             if (log) fprintf(stderr, "autotune fused layers 0+1 %dx%d: R %d  %.1f us (apart %.1f us)\n", k0.W, k0.H, R,
                              1e3 * ms / reps, 1e3 * (best_ms[0] + best_ms[1]) / reps);
             if (ms < best) {

@@ -32,3 +32,36 @@ r.render(VIEW, INTR, W, H, 2, 1.0)
 assert get("unordered") == 0, "fp8 frame"
 assert get("launches") > 40
 """)
+
+
+def test_a_frame_that_gave_up_waiting_is_reported_to_its_own_caller(run):  # noqa: F811
+    """Contexts share no error word: a frame whose kernels' bounded waits ran out fails the call
+    that waits for it (also a served request), and no other context's."""
+    run(r"""
+for prec, kernel in (("fp32", b"k_conv_split"), ("bf16", b"k_conv_halo")):
+    a, b = renderer(prec=prec), renderer(prec=prec)
+    out = Dev(12 * W * H)
+    fk.fk_give_up(kernel, 6)
+    assert status(a.render, VIEW, INTR, W, H, 2, 1.0, out=out) == 0   # returns without waiting
+    fk.fk_give_up(b"", 0)
+    assert status(b.render, VIEW, INTR, W, H, 2, 1.0) == 0, prec      # another context's frame is fine
+    assert status(a.render, VIEW, INTR, W, H, 2, 1.0) == -5, prec     # the next call of a that waits
+    assert status(a.render, VIEW, INTR, W, H, 2, 1.0) == 0, prec
+    a.serve_start(max_batch=2, slots=2)
+    def served():
+        res = np.empty((H, W, 3), np.float32)
+        t = a.submit(VIEW, INTR, W, H, 2, 1.0)
+        while True:
+            try:
+                if a.poll(t, res)[1] is not None:
+                    return 0
+            except lnr.LnrError as e:
+                return e.status
+    fk.fk_give_up(kernel, 6)
+    assert served() == -5, prec
+    fk.fk_give_up(b"", 0)
+    assert served() == 0, prec
+    assert status(b.render, VIEW, INTR, W, H, 2, 1.0) == 0, prec
+    a.serve_stop()
+    a.close(), b.close()
+""")
