@@ -44,8 +44,6 @@
 // first set is there when a chunk ends).  Holding the planes and passing the weights instead
 // was slower (128 channels: 178 against 141 us).  Every wait is bounded, as in conv_tc.cu.
 #include <cstring>
-#include <mutex>
-#include <set>
 #include <type_traits>
 
 #include "tc_ptx.h"
@@ -503,13 +501,7 @@ void pick_tile(const ConvLayer& L, int NT, int B, int W, int H, int num_sms, int
 }
 
 void launch(void (*kern)(SParams), const SParams& p, int grid, size_t smem, cudaStream_t st, TcState& tc) {
-    static std::mutex mu;
-    static std::set<const void*> done;
-    {
-        std::lock_guard<std::mutex> g(mu);
-        if (done.insert((const void*)kern).second)
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    }
+    tc_allow_smem((const void*)kern);
     kern<<<grid, kSplitThreads, smem, st>>>(p);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) tc.host_err = 9;

@@ -1389,8 +1389,7 @@ static void tc_conv_generic(const ConvLayer& L, const void* src0, const void* sr
     const size_t smem = 1024 + (size_t)p.stages * p.stage_bytes + p.xch_bytes + 8 * (2 * p.stages + 6) + 16;
     const int grid = std::min(p.ntiles, tc.num_sms);
     if (tc.host_err || !L.wtc) return;
-    static std::once_flag once;
-    std::call_once(once, [] { cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); });
+    tc_allow_smem((const void*)k_conv_tc);
     k_conv_tc<<<grid, kThreads, smem, st>>>(p);
     count_launch();
 }
@@ -1830,13 +1829,7 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
     if (stall_once.exchange(0)) p.stall = 1;
     const int grid = std::min(p.ntiles, tc.num_sms);
     auto launch = [&](void (*kern)(HParams), int threads) {
-        static std::mutex mu;
-        static std::set<const void*> done;
-        {
-            std::lock_guard<std::mutex> g(mu);
-            if (done.insert((const void*)kern).second)
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        }
+        tc_allow_smem((const void*)kern);
         kern<<<grid, threads, smem, st>>>(p);
         count_launch();
         if (cudaGetLastError() != cudaSuccess) tc.host_err = 9;  // a launch that did not start: reported, never silent
@@ -1954,13 +1947,7 @@ bool tc_enc0_fused(const ConvLayer& L0, const ConvLayer& L1, const void* in, voi
     const size_t smem = 1024 + (size_t)p.act_off + 2 * p.act_bytes + 8 * (2 * p.stages + 14) + 16;
     const int grid = std::min(p.ntiles, tc.num_sms);
     auto launch = [&](void (*kern)(FParams)) {
-        static std::mutex mu;
-        static std::set<const void*> done;
-        {
-            std::lock_guard<std::mutex> g(mu);
-            if (done.insert((const void*)kern).second)
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        }
+        tc_allow_smem((const void*)kern);
         kern<<<grid, kFuseThreads, smem, st>>>(p);
         count_launch();
         if (cudaGetLastError() != cudaSuccess) tc.host_err = 9;
@@ -2111,6 +2098,17 @@ std::vector<TcConfig> tc_candidates(const ConvLayer& L, lnr_precision prec) {
             }
         }
     return out;
+}
+
+void tc_allow_smem(const void* kernel) {
+    static std::mutex mu;
+    static std::set<std::pair<int, const void*>> done;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> g(mu);
+    if (done.count({dev, kernel})) return;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess)
+        done.insert({dev, kernel});
 }
 
 cudaError_t TcState::ensure(int sms) {

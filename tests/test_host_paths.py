@@ -65,3 +65,23 @@ for prec, kernel in (("fp32", b"k_conv_split"), ("bf16", b"k_conv_halo")):
     a.serve_stop()
     a.close(), b.close()
 """)
+
+
+def test_every_precision_runs_on_a_second_device(run):  # noqa: F811
+    """A kernel's shared-memory allowance belongs to a device, as do an SM count and the buffers
+    that a launch points to: contexts on two devices of one process, results left on the device."""
+    run(r"""
+for device in (0, 1, 0):
+    r = renderer(device)
+    for prec in ("fp32", "bf16", "fp8"):
+        if prec == "fp8":
+            r.calibrate(VIEW, INTR, W, H, 2, 1.0)
+        r.set_precision(prec)
+        for _ in range(4):                       # eager, captured, replayed
+            r.render(VIEW, INTR, W, H, 2, 1.0, out=Dev(12 * W * H))
+        assert get("refused") == 0, (device, prec)
+        assert get("foreign") == 0, (device, prec)
+        r.render(VIEW, INTR, W, H, 2, 1.0)
+    r.close()
+assert get("conv_split") > 0 and get("conv_halo") > 0
+""")
