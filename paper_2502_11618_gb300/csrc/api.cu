@@ -307,6 +307,10 @@ cudaError_t run_frame(lnr_ctx* c, Workspace& ws, lnr_precision prec, bool use_gr
             enqueue_frame(c, ws, ws.stream, -1, prec, false);
             e = cudaStreamEndCapture(ws.stream, &g);
         }
+        if (e == cudaSuccess && ws.tc.host_err) {  // a launch is missing: no graph of it; the caller reports it
+            cudaGraphDestroy(g);
+            return cudaSuccess;
+        }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
         if (g) cudaGraphDestroy(g);
         if (e != cudaSuccess) {  // capture not possible on this stream: stay eager
@@ -336,6 +340,8 @@ static void read_timing(lnr_ctx* c, Workspace& ws) {
 }
 
 static lnr_status finish_output(lnr_ctx* c, Workspace& ws, float* out, size_t nfloat, int on_device) {
+    // a launch that was refused is this call's error, wherever its output goes
+    if (const int h = ws.tc.take_host()) return fail(c, tc_error_status(h), tc_error_text(h));
     cudaError_t e = cudaSuccess;
     if (out != ws.out_ptr)  // else the U-Net wrote the caller's device buffer directly
         e = cudaMemcpyAsync(out, ws.out.p, nfloat * 4, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -830,6 +836,7 @@ lnr_status lnr_calibrate_batch(lnr_ctx* c, int nviews, const lnr_view* view, con
     ws.allow_fuse = true;
     cudaError_t e = cudaStreamSynchronize(ws.stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "calibration frame");
+    if (const int w = ws.tc.take()) return fail(c, tc_error_status(w), "calibration frame: " + tc_error_text(w));
     return unet_calibrate_fp8(c, ws);
 }
 

@@ -2124,9 +2124,14 @@ void TcState::release() {
     err = nullptr;
 }
 
-int TcState::take() {
-    int code = host_err;
+int TcState::take_host() {
+    const int code = host_err;
     host_err = 0;
+    return code;
+}
+
+int TcState::take() {
+    int code = take_host();
     if (!err) return code;
     if (!code) code = *static_cast<volatile int*>(err);
     *static_cast<volatile int*>(err) = 0;

@@ -142,6 +142,7 @@ struct TcState {
     int host_err = 0;    // on the host: 4 tensor map, 8 no FP8 configuration, 9 launch refused
     cudaError_t ensure(int sms);
     void release();
+    int take_host();  // host_err, then cleared: known as soon as the frame's launches have been made
     int take();  // the error since the last call, 0 none; the workspace's stream has been waited for
 };
 

@@ -158,6 +158,7 @@ struct Server {
     // stats
     uint64_t n_done = 0, n_launch = 0, max_b = 0, peak_bytes = 0, peak_alloc = 0, peak_busy = 0;
     std::string err;
+    std::string launch_err;  // the scheduler thread's
 
     void loop();
     bool launch(Slot& s, std::vector<uint64_t>& batch, size_t need);
@@ -214,6 +215,7 @@ bool Server::launch(Slot& s, std::vector<uint64_t>& batch, size_t need) {
         H = r0.H;
         nlev = r0.nlev;
     }
+    launch_err.clear();
     make_room(s, need);
     if (prepare_views(c, s.ws, B, views.data(), intr.data(), W, H, nlev, fs.data(), prec) != LNR_OK) return false;
     {
@@ -223,6 +225,10 @@ bool Server::launch(Slot& s, std::vector<uint64_t>& batch, size_t need) {
         peak_alloc = std::max<uint64_t>(peak_alloc, held);
     }
     if (run_frame(c, s.ws, prec, true) != cudaSuccess) return false;
+    if (const int h = s.ws.tc.take_host()) {
+        launch_err = tc_error_text(h);
+        return false;
+    }
     const size_t per = (size_t)W * H * 3;
     for (int i = 0; i < B; ++i) {
         float* dst;
@@ -313,7 +319,7 @@ void Server::loop() {
                     reqs[tk].done = true;
                     reqs[tk].status = LNR_E_CUDA;
                 }
-                err = c->err.empty() ? "launch failed" : c->err;
+                err = !launch_err.empty() ? launch_err : c->err.empty() ? "launch failed" : c->err;
                 s.busy = false;
             } else {
                 ++n_launch;

@@ -85,3 +85,55 @@ for device in (0, 1, 0):
     r.close()
 assert get("conv_split") > 0 and get("conv_halo") > 0
 """)
+
+
+def test_a_refused_launch_fails_the_call_that_made_it(run):  # noqa: F811
+    """Whatever the call: into host or device memory, eager, captured or replayed, timed, served,
+    calibration, a shard's frame.  Once launches succeed again, so do the calls, and no graph
+    without the refused launch is kept."""
+    run(r"""
+for prec, kernel in (("fp32", b"k_conv_split"), ("bf16", b"k_conv_halo")):
+    keys, rgba = Dev(8 * W * H), Dev(4 * W * H)
+    for runs in range(3):                        # eager, eager, captured
+        for host in (False, True):
+            a = renderer(prec=prec)
+            out = None if host else Dev(12 * W * H)
+            for _ in range(2 * runs):            # two view blocks in turn, each with its graph
+                a.render(VIEW, INTR, W, H, 2, 1.0, out=out)
+            fk.fk_refuse(kernel)
+            assert status(a.render, VIEW, INTR, W, H, 2, 1.0, out=out) == -4, (prec, runs, host)
+            fk.fk_refuse(b"")
+            for k in range(8):
+                convs = get("conv_split") + get("conv_halo")
+                graphs = get("graphs")
+                assert status(a.render, VIEW, INTR, W, H, 2, 1.0, out=out) == 0
+                if k == 0:                       # launched anew, not a graph without the launch
+                    assert get("conv_split") + get("conv_halo") > convs
+            assert get("graphs") > graphs
+            a.close()
+    a = renderer(prec=prec)
+    b = renderer(prec=prec)
+    fk.fk_refuse(kernel)
+    a.set_timing(True)
+    assert status(a.render, VIEW, INTR, W, H, 2, 1.0, out=Dev(12 * W * H)) == -4
+    a.set_timing(False)
+    assert status(a.shard_finish, VIEW, INTR, W, H, 2, 1.0, keys, rgba, out=Dev(12 * W * H)) == -4
+    if prec == "bf16":
+        assert status(a.calibrate, VIEW, INTR, W, H, 2, 1.0) == -4
+    a.serve_start(max_batch=2, slots=2)
+    t = a.submit(VIEW, INTR, W, H, 2, 1.0)
+    def poll():
+        while True:
+            try:
+                if a.poll(t, np.empty((H, W, 3), np.float32))[1] is not None:
+                    return 0
+            except lnr.LnrError as e:
+                return e.status
+    assert poll() == -4
+    fk.fk_refuse(b"")
+    t = a.submit(VIEW, INTR, W, H, 2, 1.0)
+    assert poll() == 0
+    a.serve_stop()
+    assert status(b.render, VIEW, INTR, W, H, 2, 1.0) == 0
+    a.close(), b.close()
+""")
