@@ -22,6 +22,7 @@ lnr_status fail(lnr_ctx* c, lnr_status s, const std::string& msg) {
 }
 
 lnr_status cuda_fail(lnr_ctx* c, cudaError_t e, const char* where) {
+    cudaGetLastError();  // reported here: the next call that asks the runtime does not find it again
     return fail(c, e == cudaErrorMemoryAllocation ? LNR_E_OOM : LNR_E_CUDA,
                 std::string(where) + ": " + cudaGetErrorString(e));
 }
@@ -884,7 +885,6 @@ lnr_status lnr_probe_atomic_rate(lnr_ctx* c, uint64_t n_slots, uint64_t n_ops, i
     Workspace& ws = c->ws;
     cudaError_t e = cudaStreamSynchronize(ws.stream);
     if (!e) e = probe_atomic_rate(n_slots, n_ops, coherent != 0, c->num_sms, ws.stream, ops_per_s);
-    if (e == cudaErrorMemoryAllocation) return fail(c, LNR_E_OOM, "atomic probe buffer");
     if (e != cudaSuccess) return cuda_fail(c, e, "atomic probe");
     return LNR_OK;
 }

@@ -45,7 +45,10 @@ struct PinnedPool {
             return p;
         }
         void* p = nullptr;
-        if (cudaMallocHost(&p, bytes) != cudaSuccess) return nullptr;
+        if (cudaMallocHost(&p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
         return static_cast<float*>(p);
     }
     void put(float* p, size_t bytes) { free_.emplace(bytes, p); }

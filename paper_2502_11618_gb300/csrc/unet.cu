@@ -443,11 +443,13 @@ lnr_status unet_prepare(lnr_ctx* c) {
         if (e != cudaSuccess) return cuda_fail(c, e, "U-Net weight upload");
     if (u.head_w) cudaFree(u.head_w);
     if (u.head_b) cudaFree(u.head_b);
-    if (cudaMalloc(&u.head_w, u.head_wh.size() * 4) || cudaMalloc(&u.head_b, u.head_bh.size() * 4))
-        return fail(c, LNR_E_OOM, "U-Net head upload");
+    u.head_w = u.head_b = nullptr;
+    cudaError_t e;
+    if ((e = cudaMalloc(&u.head_w, u.head_wh.size() * 4)) || (e = cudaMalloc(&u.head_b, u.head_bh.size() * 4)))
+        return cuda_fail(c, e, "U-Net head upload");
     cudaMemcpy(u.head_w, u.head_wh.data(), u.head_wh.size() * 4, cudaMemcpyHostToDevice);
     cudaMemcpy(u.head_b, u.head_bh.data(), u.head_bh.size() * 4, cudaMemcpyHostToDevice);
-    cudaError_t e = cudaDeviceSynchronize();
+    e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(c, e, "U-Net upload");
     return LNR_OK;
 }

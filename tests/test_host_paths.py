@@ -137,3 +137,36 @@ for prec, kernel in (("fp32", b"k_conv_split"), ("bf16", b"k_conv_halo")):
     assert status(b.render, VIEW, INTR, W, H, 2, 1.0) == 0
     a.close(), b.close()
 """)
+
+
+def test_a_failed_call_leaves_no_error_for_the_next(run):  # noqa: F811
+    """An allocation that fails is that call's error alone: the same context's and another one's
+    next calls succeed."""
+    run(r"""
+for prec in ("fp32", "bf16"):
+    a, b = renderer(prec=prec), renderer(prec=prec)
+    failed = 0
+    for k in range(1, 100):
+        B = 8 * k                                # every buffer has to grow
+        fk.fk_fail_alloc(k)
+        st = status(a.render_batch, [VIEW] * B, INTR, W, H, 2, 1.0)
+        fk.fk_fail_alloc(0)
+        if st == 0:
+            break
+        failed += 1
+        assert st == -3, st
+        assert status(b.render, VIEW, INTR, W, H, 2, 1.0) == 0, k
+        assert status(a.render, VIEW, INTR, W, H, 2, 1.0) == 0, k
+    assert failed > 10, failed
+    for k in range(1, 100):
+        fk.fk_fail_alloc(k)
+        st = status(a.set_unet, CH, synth.unet_weights(CH, seed=1), prec)
+        fk.fk_fail_alloc(0)
+        if st == 0:
+            break
+        assert st == -3 and status(b.render, VIEW, INTR, W, H, 2, 1.0) == 0, k
+        assert status(a.render, VIEW, INTR, W, H, 2, 1.0) == -2
+    assert status(a.render, VIEW, INTR, W, H, 2, 1.0) == 0
+    assert k > 5
+    a.close(), b.close()
+""")
