@@ -85,14 +85,16 @@ const char* lnr_last_error(lnr_ctx* ctx);
 
 /* Upload a cloud (Sec. 1: merged multi-scanner coloured points).  xyz: n x 3 FP64 world
  * coordinates; rgb: n x 3 uint8; scan_id: n uint8 source-scanner index (nullable: 0).
- * Invalidates any grid built before.  n must be in [1, 2^32 - 1]. */
+ * Invalidates any grid built before; after LNR_E_OOM or LNR_E_CUDA no cloud is loaded.  n must be
+ * in [1, 2^32 - 1]. */
 lnr_status lnr_load_cloud(lnr_ctx* ctx, const double* xyz, const uint8_t* rgb,
                           const uint8_t* scan_id, uint64_t n);
 
 /* Uniform-grid partition of the loaded cloud (Sec. 1; Sec. 3, "Point Cloud
  * Projection"), built on the device: grid origin g0 = floor(min/cell)*cell, stable
  * counting sort of the points by cell id (k*dy + j)*dx + i, and per point an FP32 offset to
- * its cell's FP64 origin.  cell_size > 0; at most 2^31 cells. */
+ * its cell's FP64 origin.  cell_size > 0; at most 2^31 cells.  LNR_E_ARG leaves an older grid as it
+ * was, LNR_E_OOM or LNR_E_CUDA leaves none. */
 lnr_status lnr_build_grid(lnr_ctx* ctx, double cell_size);
 
 /* Grid summary: out_g0[3] (FP64 origin), out_dims[3] (cells per axis); nullable each. */

@@ -428,6 +428,7 @@ lnr_status lnr_load_cloud(lnr_ctx* c, const double* xyz, const uint8_t* rgb, con
         if (!std::isfinite(xyz[i])) return fail(c, LNR_E_ARG, "non-finite coordinate");
     cudaError_t e;
     c->grid_ok = false;
+    c->n = 0;  // until all of it is on the device: a failure leaves no cloud
     DBuf bytes;  // colours, then scanner ids, as they come
     if ((e = c->xyz.ensure(24 * n)) || (e = c->rgbs_in.ensure(4 * n)) || (e = bytes.ensure((scan_id ? 4 : 3) * n)))
         return cuda_fail(c, e, "cloud upload");
@@ -458,6 +459,7 @@ static lnr_status build_grid_in(lnr_ctx* c, double cell, const double g0[3], con
         total *= (double)dims[a];
     }
     if (total > 2147483647.0) return fail(c, LNR_E_ARG, "too many cells (> 2^31)");
+    c->grid_ok = false;  // until it is built: from here on the old one is gone
     std::memcpy(c->g0, g0, sizeof(c->g0));
     std::memcpy(c->dims, dims, sizeof(c->dims));
     c->cell = cell;

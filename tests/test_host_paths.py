@@ -170,3 +170,44 @@ for prec in ("fp32", "bf16"):
     assert k > 5
     a.close(), b.close()
 """)
+
+
+def test_a_failed_upload_or_grid_build_leaves_no_usable_cloud(run):  # noqa: F811
+    """Every allocation of a load and of a grid build fails once: what needs the cloud or the grid
+    then answers LNR_E_STATE until a load and a build succeed.  Refused arguments change nothing."""
+    run(r"""
+frame = lambda r: status(r.render, VIEW, INTR, W, H, 2, 1.0)
+r = renderer()
+assert frame(r) == 0
+assert status(r.build_grid_frame, 0.5, [0, 0, 0], [0, 1, 1]) == -1 and frame(r) == 0
+assert status(r.build_grid, 0.0) == -1 and frame(r) == 0
+assert status(r.load_cloud, np.full((1, 3), np.nan), np.zeros((1, 3))) == -1 and frame(r) == 0
+failed, cells, n = 0, 4, 1000
+for what in ("grid", "cloud"):
+    for k in range(1, 100):
+        cells, n = cells + 3, n + 5000           # every buffer has to grow
+        if what == "grid":
+            r.load_cloud(*cloud(n))
+            r.build_grid(0.5)
+            fk.fk_fail_alloc(k)
+            st = status(r.build_grid_frame, 0.5, [0, 0, 0], [cells, cells, cells])
+        else:
+            fk.fk_fail_alloc(k)
+            st = status(r.load_cloud, *cloud(n))
+        fk.fk_fail_alloc(0)
+        if st == 0:
+            break
+        failed += 1
+        assert st == -3
+        assert frame(r) == -2, (what, k)
+        assert status(r.grid_info) == -2
+        assert status(r.serve_start) == -2
+        assert status(r.render_stage, VIEW, INTR, W, H, 2, 1.0, 0) == -2
+        if what == "cloud":
+            assert status(r.build_grid, 0.5) == -2, k
+            assert status(r.build_grid_frame, 0.5, [0, 0, 0], [2, 2, 2]) == -2
+            r.load_cloud(*cloud(10))
+        r.build_grid(0.5)
+        assert frame(r) == 0
+assert failed >= 4, failed
+""")
