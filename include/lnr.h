@@ -56,7 +56,8 @@ typedef struct {
 } lnr_intrinsics;
 
 /* U-Net shape: `levels` resolution levels with ch[l] channels, in_ch = 5 (RGBDA),
- * out_ch = 3 (RGB); has_bn = 1 when the weight file carries batch-norm statistics for the
+ * out_ch = 3 (RGB; a network with 1 or 2 outputs writes that many floats a pixel, packed, wherever a
+ * result is said to hold 3, and leaves the rest of the buffer as it was); has_bn = 1 when the weight file carries batch-norm statistics for the
  * encoder convolutions. */
 typedef struct {
     int levels;

@@ -139,6 +139,7 @@ class Renderer:
         s = None if stream is None else C.c_void_p(int(stream))
         self._check(self._L.lnr_create(C.byref(self._c), int(device), s))
         self.levels = None
+        self.out_ch = 3
 
     def _check(self, status):
         if status != 0:
@@ -184,10 +185,11 @@ class Renderer:
                                                C.c_void_p(keys_dev.data_ptr()), C.c_void_p(rgba_dev.data_ptr())))
 
     def shard_finish(self, view, intr, W, H, n_levels, fs, keys_dev, rgba_dev, out=None):
-        """The frame from the whole cloud's keys and colours (device tensors); (H, W, 3)."""
+        """The frame from the whole cloud's keys and colours (device tensors); (H, W, 3)
+        (out_ch of the network in place of 3)."""
         host = out is None
         if host:
-            out = np.empty((H, W, 3), np.float32)
+            out = np.empty((H, W, self.out_ch), np.float32)
         ptr = _ptr(out) if host else C.c_void_p(out.data_ptr())
         self._check(self._L.lnr_shard_finish(self._c, C.byref(make_view(view)), C.byref(make_intr(intr)), W, H,
                                               n_levels, float(fs), C.c_void_p(keys_dev.data_ptr()),
@@ -210,6 +212,7 @@ class Renderer:
         self._check(self._L.lnr_set_unet(self._c, C.byref(d), _ptr(w), w.size,
                                          PRECISIONS.get(precision, precision)))
         self.levels = len(ch)
+        self.out_ch = int(out_ch)
 
     def calibrate(self, view, intr, W, H, n_levels, fs):
         """Static E4M3 scales from BF16 frames; enables the FP8 precision.  `view` may be a
@@ -258,7 +261,7 @@ class Renderer:
             self._check(self._L.lnr_render(self._c, C.byref(make_view(view)), C.byref(make_intr(intr)),
                                            W, H, n_levels, float(fs), dp, 1))
             return out
-        res = np.empty((H, W, 3), np.float32) if out is None else out
+        res = np.empty((H, W, self.out_ch), np.float32) if out is None else out
         self._check(self._L.lnr_render(self._c, C.byref(make_view(view)), C.byref(make_intr(intr)),
                                        W, H, n_levels, float(fs), _ptr(res), 0))
         return res
@@ -275,7 +278,7 @@ class Renderer:
             self._check(self._L.lnr_render_batch(self._c, n, C.cast(va, C.c_void_p), C.cast(ia, C.c_void_p),
                                                  W, H, n_levels, _ptr(fsa), dp, 1))
             return out
-        res = np.empty((n, H, W, 3), np.float32) if out is None else out
+        res = np.empty((n, H, W, self.out_ch), np.float32) if out is None else out
         self._check(self._L.lnr_render_batch(self._c, n, C.cast(va, C.c_void_p), C.cast(ia, C.c_void_p),
                                              W, H, n_levels, _ptr(fsa), _ptr(res), 0))
         return res

@@ -548,7 +548,7 @@ lnr_status lnr_shard_finish(lnr_ctx* c, const lnr_view* view, const lnr_intrinsi
     s = prepare_views(c, ws, 1, view, in, W, H, nlev, &fs, c->prec);
     if (s != LNR_OK) return s;
     enqueue_from_keys(c, ws, ws.stream, keys, rgba, -1, c->prec);
-    const size_t bytes = 12 * (size_t)W * H;
+    const size_t bytes = sizeof(float) * c->unet.out_ch * (size_t)W * H;
     cudaError_t e = cudaMemcpyAsync(out, ws.out.p, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                                     ws.stream);
     if (!e) e = cudaStreamSynchronize(ws.stream);
@@ -571,7 +571,8 @@ lnr_status lnr_set_unet(lnr_ctx* c, const lnr_unet_desc* d, const float* w, size
     if (!c) return LNR_E_ARG;
     if (!d || !w) return fail(c, LNR_E_ARG, "null descriptor or weights");
     if (d->levels < 1 || d->levels > kMaxUnetLevels) return fail(c, LNR_E_ARG, "levels outside [1, 8]");
-    if (d->in_ch != 5 || d->out_ch < 1 || d->out_ch > 4) return fail(c, LNR_E_ARG, "in_ch must be 5, out_ch in [1, 4]");
+    // the frame buffers, the library's and the callers', hold three floats a pixel
+    if (d->in_ch != 5 || d->out_ch < 1 || d->out_ch > 3) return fail(c, LNR_E_ARG, "in_ch must be 5, out_ch in [1, 3]");
     if (prec < LNR_FP32 || prec > LNR_FP8) return fail(c, LNR_E_ARG, "bad precision");
     for (int l = 0; l < d->levels; ++l)
         if (d->ch[l] < 16 || d->ch[l] > 256 || d->ch[l] % 16) return fail(c, LNR_E_ARG, "channels must be multiples of 16 in [16, 256]");
@@ -712,7 +713,7 @@ lnr_status lnr_render_batch(lnr_ctx* c, int nviews, const lnr_view* views, const
         cudaError_t e = run_frame(c, ws, c->prec, true);
         if (e != cudaSuccess) return cuda_fail(c, e, "render launch");
     }
-    return finish_output(c, ws, out, (size_t)nviews * W * H * 3, on_device);
+    return finish_output(c, ws, out, (size_t)nviews * W * H * c->unet.out_ch, on_device);
 }
 
 lnr_status lnr_render(lnr_ctx* c, const lnr_view* view, const lnr_intrinsics* in, int W, int H, int nlev, float fs,

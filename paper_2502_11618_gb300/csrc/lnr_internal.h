@@ -161,7 +161,7 @@ struct Workspace {
     DBuf pyr_m, pyr_u;                      // min-pooled and upsampled levels (all levels)
     DBuf u0;                                // float [B][P] kept depth (stage tap)
     DBuf act[4 * kMaxUnetLevels + 2];       // U-Net activations; [4 * kMaxUnetLevels] = U-Net input
-    DBuf out;                               // float [B][P][3]
+    DBuf out;                               // float [B][P][out_ch], sized for 3
     float* out_ptr = nullptr;               // U-Net output of the next frame: a caller's device buffer, or null for out
     TcState tc;
     bool allow_fuse = true;                 // false: every conv runs apart (the FP8 calibration frame reads every output)

@@ -137,7 +137,7 @@ struct ServeReq {
     double t_submit = 0, t_done = 0;
     bool done = false;
     lnr_status status = LNR_OK;
-    float* host = nullptr;  // pinned result, H*W*3 floats
+    float* host = nullptr;  // pinned result, H*W*out_ch floats
     size_t bytes = 0;
     float* user = nullptr;  // lnr_submit_into: the caller's destination
     bool user_pinned = false;  // ... page-locked: the result is copied straight into it
@@ -232,7 +232,7 @@ bool Server::launch(Slot& s, std::vector<uint64_t>& batch, size_t need) {
         launch_err = tc_error_text(h);
         return false;
     }
-    const size_t per = (size_t)W * H * 3;
+    const size_t per = (size_t)W * H * c->unet.out_ch;
     for (int i = 0; i < B; ++i) {
         float* dst;
         {

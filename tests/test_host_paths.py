@@ -211,3 +211,46 @@ for what in ("grid", "cloud"):
         assert frame(r) == 0
 assert failed >= 4, failed
 """)
+
+
+def test_outputs_are_as_large_as_the_network_writes_them(run):  # noqa: F811
+    """A fourth output would be written past the frame buffers, which hold three floats a pixel:
+    refused, the network before it stays.  One or two outputs fill that many floats a pixel and
+    nothing after them, whichever call delivers them."""
+    run(r"""
+def weights(o): return synth.unet_weights(CH, seed=1, out_ch=o)
+for prec in ("fp32", "bf16"):
+    r = renderer(prec=prec)
+    for o in (0, 4, 5):
+        assert status(r.set_unet, CH, weights(max(o, 1)), prec, out_ch=o) == -1, o
+    assert status(r.render, VIEW, INTR, W, H, 2, 1.0) == 0
+    for o in (1, 2, 3):
+        r.set_unet(CH, weights(o), prec, out_ch=o)
+        P = W * H
+        def check(buf, n):
+            assert (buf[:n] == 0.0).all() and (buf[n:] == -7.0).all(), (prec, o)
+        def fresh(views=1):
+            return np.full(views * P * 3, -7.0, np.float32)
+        buf = fresh()
+        r.render(VIEW, INTR, W, H, 2, 1.0, out=buf)
+        check(buf, o * P)
+        buf = fresh(4)
+        r.render_batch([VIEW] * 4, INTR, W, H, 2, 1.0, out=buf)
+        check(buf, 4 * o * P)
+        buf = fresh()
+        assert fk.lnr_shard_finish(r._c, ctypes.byref(_lib.make_view(VIEW)), ctypes.byref(_lib.make_intr(INTR)), W, H, 2,
+                                   ctypes.c_float(1.0), ctypes.c_void_p(Dev(8 * P).data_ptr()),
+                                   ctypes.c_void_p(Dev(4 * P).data_ptr()), _lib._ptr(buf), 0) == 0
+        check(buf, o * P)
+        assert r.render(VIEW, INTR, W, H, 2, 1.0).shape == (H, W, o)
+        assert r.render_batch([VIEW] * 2, INTR, W, H, 2, 1.0).shape == (2, H, W, o)
+        r.serve_start(max_batch=4, slots=2)
+        bufs = [fresh() for _ in range(6)]
+        tickets = [r.submit_into(VIEW, INTR, W, H, 2, 1.0, b) for b in bufs]
+        while tickets:
+            tickets = [t for t in tickets if r.poll(t)[1] is None]
+        for b in bufs:
+            check(b, o * P)
+        r.serve_stop()
+    r.close()
+""")
