@@ -442,7 +442,9 @@ cudaError_t grid_build(lnr_ctx* c, cudaStream_t st) {
     f.inv = 1.0 / c->cell;
     int ex;
     f.divide = !std::isnormal(f.inv);
-    const bool power = std::frexp(c->cell, &ex) == 0.5 && !f.divide;
+    // The change of exponent needs normal cells (a zero's exponent field stands for 2^-1023, the
+    // size of a subnormal cell) that leave an overflown difference past every index.
+    const bool power = std::frexp(c->cell, &ex) == 0.5 && !f.divide && std::isnormal(c->cell) && ex <= 900;
     f.log2_cell = ex - 1;
     const uint64_t nblocks = (n + kTile - 1) / kTile, nog = (uint64_t)c->dims[0] + c->dims[1] + c->dims[2];
     const bool table = nog <= 65536;
