@@ -308,7 +308,7 @@ lnr_status lnr_probe_atomic_rate(lnr_ctx* ctx, uint64_t n_slots, uint64_t n_ops,
  * d_kept:  device float [H*W] output, the kept depth, +inf where empty or filtered out.
  * n_levels, fs: as lnr_render.  cuda_stream: cudaStream_t (NULL = legacy default stream).
  * Runs on the current CUDA device and allocates nothing: the pyramid lives in a fixed
- * 12 MiB device array inside the library (held by every GPU that loads it until exit),
+ * 6 MiB device array inside the library (held by every GPU that loads it until exit),
  * enough for images up to about 2560 x 1440 at 6 levels; larger images return LNR_E_ARG.
  * The first call on a device looks up that array's address; make it before any stream
  * capture.  Calls whose work overlaps on the GPU share the array and race; order them.

@@ -869,10 +869,11 @@ void launch_unet_in_extract(const void* unet_in, int kind, float* out5, int64_t 
 namespace lnr {
 namespace {
 
-// 3 Mi floats (12 MiB): the min-pooled levels M1..Mn.  Images whose min-pooled and upsampled
-// levels together would not fit are refused (2560 x 1440 with 6 levels needs about 2.5 Mi).
-constexpr size_t kStaticFilterFloats = size_t(3) << 20;
-constexpr size_t kStaticViewFloats = 64;
+// 1.5 Mi floats (6 MiB): the min-pooled levels M1..Mn of any image taken (2560 x 1440 with 6
+// levels: 1.25 Mi).  The limit on them dates from an array that held the upsampled levels and a
+// view's parameters, too; the same images are refused as then.
+constexpr size_t kStaticFilterFloats = size_t(3) << 19;
+constexpr size_t kStaticMaxLevels = kStaticFilterFloats - 32;  // floats of M1..Mn, at most
 
 __device__ __align__(256) float g_filter_scratch[kStaticFilterFloats];
 
@@ -1067,7 +1068,7 @@ extern "C" lnr_status lnr_filter_static(const float* d_depth, int W, int H, int 
     while ((2 << maxl) <= std::min(W, H)) ++maxl;
     if (n_levels < 0 || n_levels > std::min(maxl, kMaxLevels) || !(fs >= 0.0f)) return LNR_E_ARG;
     const size_t lev = pyramid_floats(W, H, n_levels);
-    if (kStaticViewFloats + 2 * lev > kStaticFilterFloats) return LNR_E_ARG;  // beyond the static capacity
+    if (lev > kStaticMaxLevels) return LNR_E_ARG;  // beyond the static capacity
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LNR_E_CUDA;
     float* scratch;

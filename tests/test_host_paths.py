@@ -254,3 +254,25 @@ for prec in ("fp32", "bf16"):
         r.serve_stop()
     r.close()
 """)
+
+
+def test_filter_without_allocation_takes_the_same_images(run):  # noqa: F811
+    """The images that lnr_filter_static takes: those whose levels 1..n, twice over and 64 floats,
+    come to at most 3 Mi floats."""
+    run(r"""
+def levels(w, h, n):
+    total = 0
+    for _ in range(n):
+        w, h = (w + 1) // 2, (h + 1) // 2
+        total += w * h
+    return total
+buf = Dev(64)
+p = ctypes.c_void_p(buf.data_ptr())
+taken = 0
+for w, h in [(64, 64), (1920, 1080), (2560, 1440), (4096, 4096)] + [(2048, h) for h in range(2289, 2313)]:
+    for n in range(1, 7):
+        want = 0 if 64 + 2 * levels(w, h, n) <= 3 << 20 else -1
+        taken += want == 0
+        assert fk.lnr_filter_static(p, w, h, n, ctypes.c_float(1.0), p, None) == want, (w, h, n)
+assert 18 < taken < 150, taken
+""")
