@@ -82,6 +82,7 @@ struct SParams {
     float* logits;
     int head_o;
     int* err;
+    int stall;  // 1: the MMA issuers first wait on a barrier nothing arrives on, for ~1 ms (tests)
     alignas(16) float bias[256];
     alignas(16) float head[4 * 256];  // the head's weights [4][N], zero past its outputs
 };
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_conv_split(const __grid_co
     auto t_empty = [&](int b) { return bars + 8u * (2 * SA + 2 * kBSlots + 2 + b); };
     const uint32_t drain = bars + 8u * (2 * SA + 2 * kBSlots + 4);
     const uint32_t tslot = bars + 8u * (2 * SA + 2 * kBSlots + 5);
+    const uint32_t never = bars + 8u * (2 * SA + 2 * kBSlots + 6);  // p.stall's barrier
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < SA; ++s) {
@@ -168,6 +170,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_conv_split(const __grid_co
             mbar_init(t_empty(b), kEpi);
         }
         mbar_init(drain, Sp::issuers);
+        mbar_init(never, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) tmem_alloc(tslot, p.tmem_cols);
@@ -251,7 +254,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_conv_split(const __grid_co
         int k = 0;                 // chunks issued
         uint32_t ub = 0;           // next use of the weight ring
         uint32_t as = 0, aph = 0;  // slot and phase of the plane ring
-        bool ok = true;
+        bool ok = !p.stall || mbar_wait(never, 0, kStallWaitCycles);
         for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
             int n, x0, y0, nt;
             tile_of(t, n, x0, y0, q.py, nt);
@@ -625,13 +628,14 @@ void conv_split(const ConvLayer& L, const void* src0, const void* src1, void* ou
     if (logits)
         for (int i = 0; i < head_o * N; ++i) p.head[i] = head_wh[i];
     p.err = tc.err;
+    p.stall = tc_stall_once();
     for (int i = 0; i < N; ++i) p.bias[i] = L.bf[i];
     if (!ok) {
         tc.host_err = 4;
         return;
     }
     const size_t smem = 1024 + (size_t)p.a_slots * p.a_slot + (size_t)kBSlots * p.b_slot +
-                        8 * (2 * p.a_slots + 2 * kBSlots + 6);
+                        8 * (2 * p.a_slots + 2 * kBSlots + 7);
     const int grid = std::min(p.ntiles, num_sms);
     auto go = [&](auto r, auto par, auto nt) {
         launch(k_conv_split<decltype(r)::value, decltype(par)::value, decltype(nt)::value>, p, grid, smem, st, tc);

@@ -48,7 +48,6 @@ __host__ __device__ constexpr int halo_mma_warps(int par, int r) {
 // 128 registers per thread).  12 for standard tiles and for tiles of two parity classes and
 // at most two rows, whose two issuers leave room for them.
 __host__ __device__ constexpr int halo_threads(int par, int r, int epi) { return 32 * (1 + halo_mma_warps(par, r) + epi); }
-constexpr long long kStallWaitCycles = 2000000ll;  // ~1 ms: the timeout test's wait
 constexpr int kXchStride = 33;                   // floats per row of the pooling exchange
 
 struct Seg {
@@ -1819,14 +1818,7 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
     p.head_o = head_o;
     p.err = tc.err;
     const size_t smem = 1024 + (size_t)p.stages * p.stage_bytes + stg_total + 8 * (2 * p.stages + 7) + 16;
-    // LNR_TEST_STALL_ONCE=1: the first halo launch of the process waits on a barrier nothing
-    // arrives on and gives up after ~1 ms; the others then give up after ~2 s (the test of
-    // the bounded waits and LNR_E_TIMEOUT)
-    static std::atomic<int> stall_once{[] {
-        const char* e = getenv("LNR_TEST_STALL_ONCE");
-        return e && atoi(e) == 1 ? 1 : 0;
-    }()};
-    if (stall_once.exchange(0)) p.stall = 1;
+    p.stall = tc_stall_once();
     const int grid = std::min(p.ntiles, tc.num_sms);
     auto launch = [&](void (*kern)(HParams), int threads) {
         tc_allow_smem((const void*)kern);
@@ -2098,6 +2090,17 @@ std::vector<TcConfig> tc_candidates(const ConvLayer& L, lnr_precision prec) {
             }
         }
     return out;
+}
+
+// LNR_TEST_STALL_ONCE=1: the MMA issuers of the first halo or FP32 convolution of the process
+// wait on a barrier nothing arrives on and give up after ~1 ms; the others then give up after ~2 s
+// (the tests of the bounded waits and LNR_E_TIMEOUT).
+int tc_stall_once() {
+    static std::atomic<int> left{[] {
+        const char* e = getenv("LNR_TEST_STALL_ONCE");
+        return e && atoi(e) == 1 ? 1 : 0;
+    }()};
+    return left.load(std::memory_order_relaxed) ? left.exchange(0) : 0;
 }
 
 void tc_allow_smem(const void* kernel) {

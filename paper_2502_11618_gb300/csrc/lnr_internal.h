@@ -308,6 +308,7 @@ bool tc_fused_enc0(const ConvLayer& L0, const ConvLayer& L1, lnr_precision p, co
 cudaError_t tc_prepare_fp8(ConvLayer& L);
 std::vector<uint16_t> halo_blocks(const ConvLayer& L, int sg);  // weight blocks of a K segment, as tap masks
 void tc_allow_smem(const void* kernel);  // all of an SM's shared memory for this kernel on the current device
+int tc_stall_once();       // 1 for the launch that a test of the bounded waits stalls
 bool tc_variant_forced();  // an LNR_CONV_* switch of the tests asks for one kernel variant
 
 // conv_split.cu: the FP32 network's convolutions.  Sources and outputs are [image][hi, mid,

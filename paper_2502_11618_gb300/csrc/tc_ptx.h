@@ -12,6 +12,7 @@ namespace lnr {
 namespace {
 
 constexpr long long kWaitCycles = 4000000000ll;  // ~2 s at 2 GHz
+constexpr long long kStallWaitCycles = 2000000ll;  // ~1 ms: the timeout tests' wait
 constexpr int kMmaWarps = 4;
 constexpr int kHaloW = 130;  // staged pixels per halo row
 
@@ -120,12 +121,6 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t sbo, uint32_t 
 }
 
 __device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"((uint64_t)m), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
-        : "memory");
-}
 
 // n contiguous bytes into shared memory.  A TMA box moves about one of its rows per cycle,
 // whatever their length: rows of 32 bytes come at 25 bytes per cycle and SM, rows of 64 at 50
