@@ -6,7 +6,8 @@
 //                          lo = BF16(v - hi - mid)
 // (together 24 significant bits), and a product of two of them as the six partial products
 // hi hi, hi mid, mid hi, hi lo, lo hi, mid mid; the dropped ones are near 2^-26 of the
-// product.  A convolution takes the MMAs of six BF16 ones, and these bound it: a tile's
+// product on average and at most 2^-22 of it.  (Parts have BF16's exponents: below about
+// 2^-110 a value's lowest bits are lost.)  A convolution takes the MMAs of six BF16 ones, and these bound it: a tile's
 // operand reads from shared memory (32 + n / 4 cycles an MMA of n columns) and the loads that
 // share its bandwidth.
 //
@@ -20,8 +21,14 @@
 //    registers, in FP32 rounded to nearest, while the MMAs of the next chunk run into the
 //    other half of TMEM;
 //  - hi has 7 bits and not BF16's 8, so that products have 14 and more of the sums are exact.
-// Frames against a 64-bit network (relative 2-norm): 1.0e-7 at 1920x1080, 8.5e-8 at 256x256;
-// with FP32 multiply-adds 1.9e-7 and 1.2e-7 on the same inputs.
+// Errors against a 64-bit network (relative 2-norm) depend on cloud, pose and weights.  Of six
+// pairs of frames with FP32 multiply-adds on the same inputs (the worst 2.5e-7 against 5.3e-7, the
+// best 7.5e-8 against 1.3e-7) these have 0.36 to 0.58 of the error.  Logits of a 264x136 view,
+// net 32-64-128, three seeds each, for other weights than He-normal ones (5.6e-7 to 8.8e-7 against
+// 6.1e-7 to 1.2e-6): pairs of taps that cancel to a thousandth 1.3e-6 against 3.0e-6; log-normal
+// magnitudes (sigma 3) 2.2e-7 to 9.4e-7 against 2.2e-7 to 8.8e-7; all positive, where truncations
+// add up, 2.0e-7 to 2.6e-7 against 2.0e-7 to 2.1e-7; layers scaled by 2^-100 and 2^100 in turn as
+// unscaled.
 //
 // Measured on a 1080p view with the 4-level net (before: CUDA-core kernels, bound by their
 // shared-memory operand reads): all convolutions 19.0 -> 2.4 ms.  Level 0: 107, 227 and 211
@@ -55,7 +62,7 @@ constexpr int kEpi = 8;           // epilogue warps
 constexpr int kIssuers = 2;       // MMA-issuing warps, at most
 constexpr int kSplitThreads = 32 * (1 + kIssuers + kEpi);
 constexpr int kBSlots = 4;        // weight sets: a chunk's three and the next one's first
-constexpr float kMaxAct = 3.3e38f;  // its leading part is still finite
+constexpr float kMaxAct = 3.3e38f;  // its leading part is still finite; larger activations (infinite, past FP32) count as it
 constexpr uint32_t kSmemBudget = 225u * 1024u;
 
 struct SSeg {

@@ -1532,7 +1532,9 @@ static int halo_bload(int kind, int P) { return kind == 2 ? (P == 4 ? 16 : 8) : 
 static bool halo_parity_ok(const ConvLayer& L, int P) { return P == 1 || (P >= 2 && 2 * L.cout <= 256); }
 
 // Bytes of one pipeline stage of the halo kernel for a layer at tile height R, P parity
-// classes per tile (decoder concat convs) and chunks of at most ckmax channels.
+// classes per tile (decoder concat convs) and chunks of at most ckmax channels: a bound.  The
+// upsampled operand of a single y class is staged in R + 1 rows and counted with R + 2, as it was
+// when the rules that choose a tile were measured.
 static uint32_t halo_stage_bytes(const ConvLayer& L, int R, int P, int ckmax, int esize = 2) {
     const int segC[2] = {tc_c0(L), L.cin1};
     uint32_t st = 0;
@@ -1787,7 +1789,6 @@ bool tc_conv_halo(const ConvLayer& L, const void* src0, const void* src1, void* 
     p.stg_bytes = stg_total;
     if (stg_total + 2 * p.stage_bytes > 220u * 1024u) return false;  // staging + two pipeline stages must fit
     p.stages = std::min<int>(8, (int)((220u * 1024u - stg_total) / p.stage_bytes));
-    (void)halo_stage_bytes;
     if (p.stages < 2) return false;
     if (!ok) {
         tc.host_err = 4;

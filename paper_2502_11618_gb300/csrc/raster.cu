@@ -37,7 +37,11 @@ constexpr int kSplatThreads = 256;
 // a warp) up to 1024, at most the visible points that every warp of the GPU would get, taking
 // a sixth of the cloud to be visible in each view.  A range of 1024 points is eight batches in a
 // row: with fewer ranges than warps the splat waits for those (200k points: 16.2 us with 1024,
-// 5.6 with 128; from 5M points on no difference), with many its cells are loaded less often.
+// 5.6 with 128; one 1080p view of 5M and 20M points 26.6 -> 10.1 and 22.5 -> 16.4; eight views of
+// 1M 40.9 -> 16.4), with many its cells are loaded less often.  Eight views of 10M points and
+// more have ranges of 1024, as without the rule; there two builds of the same work differ by the
+// run (20M points: 81.8 and 83.9 us, 84.0 and 92.1, 84.3 and 79.9 on three machines, with the same
+// instructions and DRAM bytes; the size as a template argument changed none of it).
 inline int splat_shift(uint64_t npoints, int nviews) {
     const uint64_t per_warp = npoints * (uint64_t)nviews / (6 * 4864);  // 152 SMs x 32 warps
     int s = 7;
@@ -760,10 +764,10 @@ size_t pyramid_floats(int W, int H, int nlev) { return pyramid_offset(W, H, nlev
 
 void launch_resolve_pyramid(const lnr_ctx* c, Workspace& ws, cudaStream_t st) {
     dim3 g((ws.W + 63) / 64, (ws.H + 63) / 64, ws.B);
-    // 1024 threads a tile when all tiles are on the GPU at once (2 to an SM): a thread's keys and
-    // colours come one round of loads after the other, four rounds instead of sixteen (256x256
-    // 11.2 -> 5.7 us, 1080p 18.4 -> 14.4); past 8 small blocks an SM, 256 threads (eight 1080p
-    // views: 81 against 93 us)
+    // 1024 threads a tile up to 8 tiles an SM (of which two are resident at a time: four waves): a
+    // thread's keys and colours come one round of loads after the other, four rounds instead of
+    // sixteen (256x256, 16 tiles, 11.2 -> 5.7 us; 1080p, 510 tiles, 18.4 -> 14.4); past that, where
+    // 8 blocks of 256 threads an SM are resident throughout, 256 (eight 1080p views: 81 against 93 us)
     const bool few = (int64_t)g.x * g.y * g.z < 8 * (int64_t)c->num_sms;
     (few ? k_resolve_pyramid<1024> : k_resolve_pyramid<256>)<<<g, few ? 1024 : 256, 0, st>>>(
         ws.keys.as<unsigned long long>(), c->rgbs.as<uint32_t>(), ws.W, ws.H,
