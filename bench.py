@@ -134,11 +134,11 @@ def peaks():
 # (8 x 1080p views, BF16): ncu DRAM counters of the 13 conv launches of a 2-view step, x 4
 # (scaled by the views processed).  It describes the conv kernels as captured: reported
 # only while their sources are unchanged.
-CONV_TRAFFIC = {"bytes_per_step": 10516.8e6,
+CONV_TRAFFIC = {"bytes_per_step": 10539.4e6,
                 "sha256": {"paper_2502_11618_gb300/csrc/conv_tc.cu":
-                           "7a9004f0b909af8054c3e420afef8d1cad3f622cb1e3cc30dd212568aa11f93e",
+                           "37708dae14fa8e19110dfbe084c7dfece29c97f42d11b58757d2bee437358881",
                            "paper_2502_11618_gb300/csrc/unet.cu":
-                           "73ac1bad49f33b6771b5bc4f2b055aa06029aa1f464c4a4de00f1f36b4621dc2"}}
+                           "202b4c25b79ac9e7984e8ed41181514f8f764595111c66502ee03f62b23ffc11"}}
 
 
 def conv_traffic():

@@ -124,8 +124,8 @@ __device__ __forceinline__ float round_f32(double v) {
 
 // Cell id of every point and the histogram of its lowest digit per radix tile.  Bound by the
 // FP64 pipe (one operation per SM and cycle): 20M points 2296 us with three divisions a point
-// and a global count per cell, 247 us with 6 operations, 123 us with 3 (POWER: the cell is a power
-// of two).
+// and a global count per cell, 247 us with 6 operations (268 with cells of 0.3 m), 123 us with 3
+// (POWER: the cell is a power of two).
 template <bool POWER>
 __global__ void __launch_bounds__(kThreads) k_cell_id(const double* __restrict__ xyz, uint64_t n, const GridFrame f,
                                                       uint32_t* __restrict__ cid, uint32_t* __restrict__ hist,
@@ -381,8 +381,8 @@ __global__ void k_pack_rgbs(const uint8_t* __restrict__ rgb, const uint8_t* __re
 // Sorted points: FP32 offsets to their cells' FP64 origins, and colours.  key and val (cell
 // and index of the point at each position) may lie in two of the output arrays: a thread reads
 // its position's before it writes there.  Bound by gathering 24 + 4 bytes from random points,
-// of which DRAM moves 64 each: 20M points 552 us (667 with the origins in FP64 per point and
-// colours in separate bytes).
+// for which DRAM reads 173 (3.6 GB in all at 20M points): 552 us (667 with the origins in FP64
+// per point and colours in separate bytes).
 __global__ void __launch_bounds__(kThreads) k_offsets(const double* __restrict__ xyz, const uint32_t* __restrict__ rgbs_in,
                                                       const uint32_t* key, const uint32_t* val, uint64_t n,
                                                       const GridFrame f, const double* __restrict__ og, float* ox, float* oy,

@@ -926,7 +926,8 @@ __global__ void __launch_bounds__(512) k_pyramid_from_depth(const float* __restr
 // coarse work, itself a third of the fine).  Positions outside the image hold the values of the
 // nearest pixel inside, as the replicated borders of the method.  One launch in place of one
 // per level, whose grids of a few blocks each took 5 us one after the other: 1920x1080 with 5
-// levels, whole call 40.9 -> 20.5 us.  Bound by its instructions (76 % of issue slots).
+// levels, whole call 40.9 -> 20.5 us.  Bound by its instructions (75 % of issue slots while a
+// block runs).
 struct FusedLevel {
     int W, H;        // level size
     const float* M;  // min-pooled level
